@@ -135,7 +135,6 @@ cudaError_t launch_cg_flush(Tf* x, const Tf* p, const RhsState* st, long long pe
   cg_flush_kernel<Tf><<<dim3((unsigned)b, (unsigned)n), 256, 0, s>>>(x, p, st, per);
   return cudaGetLastError();
 }
-template cudaError_t launch_cg_flush<float>(float*, const float*, const RhsState*, long long, int, cudaStream_t);
 template cudaError_t launch_cg_flush<double>(double*, const double*, const RhsState*, long long, int, cudaStream_t);
 
 template <typename Ti, typename To>

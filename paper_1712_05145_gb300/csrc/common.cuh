@@ -113,6 +113,26 @@ __host__ __device__ constexpr double cosm48(int m) {
 }
 __host__ __device__ constexpr double sinm48(int m) { return cosm48(12 - m); }
 
+// cos(2 pi j / 32) for j = 0..8, and cos, sin of 2 pi m / 32 for any integer m (radix 32)
+__host__ __device__ constexpr double cos32(int j) {
+  return j == 0 ? 1.0
+       : j == 1 ? 0.98078528040323044913
+       : j == 2 ? 0.92387953251128675613
+       : j == 3 ? 0.83146961230254523708
+       : j == 4 ? 0.70710678118654752440
+       : j == 5 ? 0.55557023301960222474
+       : j == 6 ? 0.38268343236508977173
+       : j == 7 ? 0.19509032201612826785
+       : 0.0;
+}
+__host__ __device__ constexpr double cosm32(int m) {
+  return ((m % 32) + 32) % 32 <= 8 ? cos32(((m % 32) + 32) % 32)
+       : ((m % 32) + 32) % 32 <= 16 ? -cos32(16 - ((m % 32) + 32) % 32)
+       : ((m % 32) + 32) % 32 <= 24 ? -cos32(((m % 32) + 32) % 32 - 16)
+       : cos32(32 - ((m % 32) + 32) % 32);
+}
+__host__ __device__ constexpr double sinm32(int m) { return cosm32(8 - m); }
+
 // v *= exp(DIR * 2 pi i * m / R), exact for multiples of a quarter turn.
 template <typename T, int R, int M, int DIR>
 __device__ __forceinline__ cx<T> twiddle_c(cx<T> v) {
@@ -126,9 +146,10 @@ __device__ __forceinline__ cx<T> twiddle_c(cx<T> v) {
   } else if constexpr (4 * m == 3 * R) {
     return mul_i<T, -DIR>(v);
   } else {
-    constexpr int q = 48 / R * m;
-    const T c = (T)cosm48(q);
-    const T s = (T)(DIR * sinm48(q));
+    static_assert(48 % R == 0 || R == 32, "no twiddle table of this radix");
+    constexpr int q = (R == 32) ? m : 48 / R * m;
+    const T c = (T)(R == 32 ? cosm32(q) : cosm48(q));
+    const T s = (T)(DIR * (R == 32 ? sinm32(q) : sinm48(q)));
     return mk<T>(v.re * c - v.im * s, v.re * s + v.im * c);
   }
 }

@@ -23,6 +23,7 @@
 #include "hierarchy.h"
 #include "plane_cluster.h"
 #include "polarization.h"
+#include "spectral_cg.h"
 #include "zcluster.h"
 #include "zsplit.h"
 #include "hom.h"
@@ -207,7 +208,15 @@ hom_status work(hom_ctx* c, int i, size_t bytes, void** out) {
 
 // partial sums one load's reducing kernel publishes at most (one per CTA)
 size_t ncta_max(const hom_ctx* c) {
-  return 6 * (size_t)std::max(c->g.n3 * std::max(1, c->g.pc_Q), c->g.split ? c->g.nrb : 0) + 64;
+  size_t m = 6 * (size_t)std::max(c->g.n3 * std::max(1, c->g.pc_Q), c->g.split ? c->g.nrb : 0);
+  if (c->fp32)   // the CG passes in Fourier space: row blocks and z tiles
+    m = std::max(m, std::max(6 * (size_t)cg_row_blocks(c->g), (size_t)cg_z_blocks(c->g)));
+  return m + 64;
+}
+
+// bytes of n loads' vectors in Fourier space (three complex FP32 components per frequency)
+size_t hat_bytes(const hom_ctx* c, int n) {
+  return (size_t)n * (size_t)cg_vector_elems(c->g) * sizeof(cx<float>);
 }
 
 // grows the per-load state, partial and load arrays to `n` loads
@@ -620,13 +629,143 @@ hom_status apply_A(hom_ctx* c, int n, const Tf* in, Tf* out, const std::vector<i
   return ls_pass<Tf, Tf, Tf>(c, n, fa, za, ia, act);
 }
 
+// Launch arguments of the FP32 CG iteration in Fourier space (spectral_cg.h)
+struct CgPass {
+  CgZArgs za{};
+  CgPlaneArgs pa{};
+  bool whole_planes = false;   // cg_plane holds a plane per CTA; else the y pass, cg_rows, the y pass
+};
+CgPass cg_pass(hom_ctx* c, cx<float>* rh, cx<float>* ph, cx<float>* xh) {
+  CgPass q;
+  int chunk;
+  cx<float>* S = spec<float>(c, &chunk);
+  CgZArgs& za = q.za;
+  za.g = c->g;
+  za.S = S;
+  za.r = rh;
+  za.p = ph;
+  za.x = xh;
+  za.st = c->d_st;
+  za.lam0 = c->lam0;
+  za.mu0 = c->mu0;
+  za.rve_loads = c->rve_loads;
+  za.c0 = c->rve_loads > 0 ? c->d_c0 : nullptr;
+  za.scale = (float)(1.0 / (double)c->g.M);
+  za.green = c->opt.green_operator;
+  za.gtab = c->d_gtab;
+  za.tw_n3 = tw<float>(c, 3);
+  za.part = part_inv(c);
+  za.cnt = cnt_inv(c);
+  za.prof = c->prof_on ? c->d_prof + 2 * HOM_KERNEL_ZPASS : nullptr;
+  CgPlaneArgs& pa = q.pa;
+  pa.g = c->g;
+  pa.S = S;
+  pa.st = c->d_st;
+  pa.phase = c->d_phase;
+  pa.mat = c->d_mat32;
+  pa.n_phase = c->nphase;
+  pa.rve_loads = c->rve_loads;
+  pa.tw_h = tw<float>(c, 0);
+  pa.tw_n1 = tw<float>(c, 1);
+  pa.tw_n2 = tw<float>(c, 2);
+  pa.part = part_fwd(c);
+  pa.cnt = cnt_fwd(c);
+  pa.prof = c->prof_on ? c->d_prof + 2 * HOM_KERNEL_PLANE_INV : nullptr;
+  q.whole_planes = c->opt.pass_mode != 2 && cg_plane_fits(c->g);
+  return q;
+}
+
+// `iters` CG iterations of the m loads from r0 on (inactive loads are skipped on the device)
+hom_status cg_iterations(hom_ctx* c, CgPass& q, int r0, int m, int iters) {
+  unsigned long long* yp = c->prof_on ? c->d_prof + 2 * HOM_KERNEL_YPASS : nullptr;
+  auto y = [&](int dir) {
+    return timed_launch(c, HOM_KERNEL_YPASS,
+                        [&] { return ypass<float>(c, q.pa.tw_n2, q.pa.S, 6, 6, m, dir, yp, c->d_st, r0); });
+  };
+  q.za.rhs0 = q.pa.rhs0 = r0;
+  for (int k = 0; k < iters; ++k) {
+    CKS(timed_launch(c, HOM_KERNEL_ZPASS, [&] { return launch_cg_z_inv(q.za, CGI_STEP, m, c->stream); }));
+    if (q.whole_planes) {
+      CKS(timed_launch(c, HOM_KERNEL_PLANE_INV, [&] { return launch_cg_plane(q.pa, m, c->stream); }));
+    } else {
+      CKS(y(+1));
+      CKS(timed_launch(c, HOM_KERNEL_PLANE_INV, [&] { return launch_cg_rows(q.pa, m, c->stream); }));
+      CKS(y(-1));
+    }
+    CKS(timed_launch(c, HOM_KERNEL_ZPASS, [&] { return launch_cg_z_fwd(q.za, CGF_STEP, m, c->stream); }));
+  }
+  return HOM_OK;
+}
+
+// One FP32 CG sweep on A d = r (Eq. cg_form) with its vectors in Fourier space, for the active loads:
+// r (real, compatible) goes to rh, CG runs until every load's device state is inactive, and the
+// correction d is added to x64.  rh, ph, xh: n loads' vectors (hat_bytes); ph may be r's buffer, which
+// is read before the first iteration writes p.  A chunk of loads runs check_every iterations before the
+// next chunk starts, so that vectors that fit the L2 cache stay there.
+hom_status cg_sweep_fourier(hom_ctx* c, int n, const float* r, cx<float>* rh, cx<float>* ph, cx<float>* xh,
+                            double* x64, std::vector<RhsState>& st, std::vector<int>& act) {
+  const std::vector<int> ran = act;
+  const int chunk = c->chunk;
+  CgPass q = cg_pass(c, rh, ph, xh);
+  auto any_of = [&](const std::vector<int>& v, int r0, int m) {
+    for (int i = r0; i < r0 + m; ++i)
+      if (v[i]) return true;
+    return false;
+  };
+  // r -> rh
+  auto fa = fwd_args<float, float>(c, FWD_COPY, 6, 6);
+  fa.in = r;
+  fa.st = c->d_st;
+  fa.S = q.za.S;
+  for (int r0 = 0; r0 < n; r0 += chunk) {
+    const int m = std::min(chunk, n - r0);
+    if (!any_of(act, r0, m)) continue;
+    fa.rhs0 = q.za.rhs0 = r0;
+    CKS((fwd_xy<float, float>(c, fa, m)));
+    CKS(timed_launch(c, HOM_KERNEL_ZPASS, [&] { return launch_cg_z_fwd(q.za, CGF_INIT, m, c->stream); }));
+  }
+  CK(cudaMemsetAsync(xh, 0, hat_bytes(c, n), c->stream));
+  bool any = true;
+  while (any) {
+    for (int r0 = 0; r0 < n; r0 += chunk) {
+      const int m = std::min(chunk, n - r0);
+      if (any_of(act, r0, m)) CKS(cg_iterations(c, q, r0, m, c->opt.check_every));
+    }
+    CKS(read_states(c, n, st));
+    any = false;
+    for (int i = 0; i < n; ++i) {
+      act[i] = st[i].active;
+      any = any || act[i];
+    }
+  }
+  // x64 += d, with the update of x that the last iteration left pending
+  for (int i = 0; i < n; ++i) st[i].active = ran[i];
+  CKS(write_states(c, st));
+  auto ia = inv_args<double, float>(c, INV_ADD, FIN_NONE, 6, 6, 6);
+  ia.S = q.za.S;
+  ia.st = c->d_st;
+  ia.out = x64;
+  for (int r0 = 0; r0 < n; r0 += chunk) {
+    const int m = std::min(chunk, n - r0);
+    if (!any_of(ran, r0, m)) continue;
+    q.za.rhs0 = ia.rhs0 = r0;
+    CKS(timed_launch(c, HOM_KERNEL_ZPASS, [&] { return launch_cg_z_inv(q.za, CGI_OUT, m, c->stream); }));
+    CKS((inv_xy<double, float>(c, ia, m)));
+  }
+  for (int i = 0; i < n; ++i) {
+    st[i].xpend = 0;
+    st[i].active = 0;
+  }
+  return HOM_OK;
+}
+
 // Autotuner (hom_options.autotune): times one operator application per candidate launch shape
 // on this handle's grid and keeps the fastest per load.  The candidates are the loads per launch
 // (1, 2, 3, 4, 6, 8, 12, ... up to the spectrum scratch's capacity, at most 12), the z stages
 // that fit (the single-CTA z pass with tiles of 2^0 .. 2^4 columns, the cluster z pass with tiles
 // of at least 32 bytes per z-plane) and, on planes above one CTA, the cluster plane passes against
 // the split x and y passes; then the split y pass's tile width.  It tunes the passes of the
-// iteration precision T.
+// iteration precision T; FP32 CG handles take their loads per launch from timed CG iterations.
 // Tuning cache (HOM_TUNE_CACHE): one line per tuned handle kind,
 //   key: n1 n2 n3 precision transform-bytes z_mode pass_mode n_rve green chunk-capacity y_mode
 //   value: chunk zc_off zc_lg ztile_lg pc_off ty_log2 zc_tma y_tma
@@ -806,6 +945,38 @@ hom_status autotune(hom_ctx* c) {
     }
     set_ytile(c->g, best_y);
     if (f32) c->y_tma = best_tma;
+  }
+  // FP32 CG iterates on its own passes (spectral_cg.h): its loads per launch are timed on them
+  if (std::is_same<T, float>::value && c->opt.scheme == HOM_CG) {
+    void* vec[3];
+    const int slot[3] = {0, 1, 3};
+    const size_t hb = hat_bytes(c, nt);
+    for (int i = 0; i < 3; ++i) {
+      CKS(work(c, slot[i], hb, &vec[i]));
+      CK(cudaMemsetAsync(vec[i], 0, hb, c->stream));
+    }
+    for (auto& s : st) s.max_iter = 1 << 30;
+    CKS(write_states(c, st));
+    CgPass q = cg_pass(c, reinterpret_cast<cx<float>*>(vec[0]), reinterpret_cast<cx<float>*>(vec[1]),
+                       reinterpret_cast<cx<float>*>(vec[2]));
+    best = 1e300;
+    for (int ck : chunks) {
+      auto sweep = [&](int iters) {
+        for (int r0 = 0; r0 < nt; r0 += ck) CKS(cg_iterations(c, q, r0, std::min(ck, nt - r0), iters));
+        return HOM_OK;
+      };
+      CKS(sweep(1));   // warm-up
+      CK(cudaEventRecord(e0, c->stream));
+      CKS(sweep(2));
+      CK(cudaEventRecord(e1, c->stream));
+      CK(cudaEventSynchronize(e1));
+      float ms = 0.0f;
+      CK(cudaEventElapsedTime(&ms, e0, e1));
+      if (ms < best) {
+        best = ms;
+        c->chunk = ck;
+      }
+    }
   }
   c->ev_pool.push_back(e0);
   c->ev_pool.push_back(e1);
@@ -999,7 +1170,8 @@ hom_status solve_system(hom_ctx* c, int n, const double* dE, const double* b64, 
                         hom_solve_info* info) {
   const bool mixed = sizeof(Tf) == sizeof(float);
   CKS(ensure_cap(c, n));
-  const size_t fb = tbytes<Tf>(c, n, 6);
+  const bool fourier = mixed && c->opt.scheme == HOM_CG;   // FP32 CG keeps its vectors in Fourier space
+  const size_t fb = fourier ? std::max(tbytes<Tf>(c, n, 6), hat_bytes(c, n)) : tbytes<Tf>(c, n, 6);
   void *vr, *vp, *vd = nullptr;
   CKS(work(c, 0, fb, &vr));
   CKS(work(c, 1, fb, &vp));
@@ -1016,16 +1188,19 @@ hom_status solve_system(hom_ctx* c, int n, const double* dE, const double* b64, 
   // the FP64 residual they restart from.
   const double kSweepGain = 1e-5, kFirstSweepTarget = 1e-4;
   const double tol_inner = (mixed && !basic) ? std::max(0.5 * tol, kFirstSweepTarget) : (mixed ? 0.5 * tol : tol);
-  // The FP32 corrections leave an incompatible part in x: CG's step lengths reach C0 / C_min
-  // along the soft phases' directions and multiply the FP32 rounding of each direction p by as
-  // much (4.4e-5 of ||b|| at 128^3 and contrast 100).  The residual form b - Gamma0 * (C : x)
+  // FP32 corrections computed on real fields (BiCGSTAB) leave an incompatible part in x: step lengths
+  // reach C0 / C_min along the soft phases' directions and multiply the FP32 rounding of each direction
+  // p by as much (4.4e-5 of ||b|| at 128^3 and contrast 100).  The residual form b - Gamma0 * (C : x)
   // does not see it, but the operator of Eq. cg_form does.  So in FP32 mode:
   //  * a sweep that aimed at the tolerance is verified with the literal residual b - A x (one
   //    FP64 pass, which sees the incompatible part); below tol the load is done;
-  //  * otherwise x is projected onto compatible fields and CG restarts from the residual of the
-  //    projected x (two FP64 passes).  The first sweep aims only at kFirstSweepTarget: the
+  //  * otherwise x is projected onto compatible fields and the scheme restarts from the residual of
+  //    the projected x (two FP64 passes).  The first sweep aims only at kFirstSweepTarget: the
   //    projection after it perturbs the residual by about the incompatible part anyway, and the
   //    later sweeps, whose corrections are small, leave a negligible incompatible part.
+  // FP32 CG keeps its vectors in Fourier space, where they are compatible by construction; what its
+  // correction adds to x is incompatible by the rounding of one FP32 transform, no more than the
+  // FP32 projection left, so its first restart needs none.
   // The polarization scheme's iterates are compatible only at the fixed point, so it takes the
   // same verification in both precisions.
   const bool project = mixed || polar;
@@ -1109,7 +1284,7 @@ hom_status solve_system(hom_ctx* c, int n, const double* dE, const double* b64, 
     }
   } else {
     CK(cudaMemsetAsync(x64, 0, tbytes<double>(c, n, 6), c->stream));
-    if (mixed) CK(cudaMemsetAsync(d, 0, fb, c->stream));
+    if (mixed && !fourier) CK(cudaMemsetAsync(d, 0, fb, c->stream));
     // initial residual r = b (x = 0)
     if (dE != nullptr) {
       auto fa = fwd_args<Tf, Tf>(c, FWD_TAU, 6, 6);
@@ -1146,36 +1321,45 @@ hom_status solve_system(hom_ctx* c, int n, const double* dE, const double* b64, 
         CKS(polar_sweep<Tf>(c, n, d, r, p, st, act));
         any = false;
       }
-      while (any) {
-        for (int k = 0; k < c->opt.check_every; ++k) {
-          auto fa = fwd_args<Tf, Tf>(c, FWD_CG, 6, 6);
-          fa.r = r;
-          fa.p = p;
-          fa.x = d;
-          fa.st = c->d_st;
-          auto za = z_args<Tf>(c, Z_GAMMA, 6, 6);
-          za.st = c->d_st;
-          auto ia = inv_args<Tf, Tf>(c, INV_CG, FIN_CG, 6, 6, 6);
-          ia.r = r;
-          ia.st = c->d_st;
-          CKS((ls_pass<Tf, Tf, Tf>(c, n, fa, za, ia, &act)));
-        }
-        CKS(read_states(c, n, st));
-        any = false;
-        bool pend = false;
-        for (int i = 0; i < n; ++i) {
-          act[i] = st[i].active;
-          any = any || act[i];
-          pend = pend || (!act[i] && st[i].xpend);
-        }
-        if (!any && pend) {
-          // the last iteration's x += alpha p, which a following forward pass would have applied
-          CK(launch_cg_flush<Tf>(d, p, c->d_st, 6 * c->g.M, n, c->stream));
-          for (int i = 0; i < n; ++i) st[i].xpend = 0;
-          CKS(write_states(c, st));
+      if constexpr (std::is_same<Tf, float>::value) {
+        if (any) {
+          CKS(cg_sweep_fourier(c, n, r, reinterpret_cast<cx<float>*>(vp), reinterpret_cast<cx<float>*>(vr),
+                               reinterpret_cast<cx<float>*>(vd), x64, st, act));
+          any = false;
         }
       }
-      if (mixed) {  // x += d, d = 0
+      if constexpr (std::is_same<Tf, double>::value) {   // CG on real fields
+        while (any) {
+          for (int k = 0; k < c->opt.check_every; ++k) {
+            auto fa = fwd_args<Tf, Tf>(c, FWD_CG, 6, 6);
+            fa.r = r;
+            fa.p = p;
+            fa.x = d;
+            fa.st = c->d_st;
+            auto za = z_args<Tf>(c, Z_GAMMA, 6, 6);
+            za.st = c->d_st;
+            auto ia = inv_args<Tf, Tf>(c, INV_CG, FIN_CG, 6, 6, 6);
+            ia.r = r;
+            ia.st = c->d_st;
+            CKS((ls_pass<Tf, Tf, Tf>(c, n, fa, za, ia, &act)));
+          }
+          CKS(read_states(c, n, st));
+          any = false;
+          bool pend = false;
+          for (int i = 0; i < n; ++i) {
+            act[i] = st[i].active;
+            any = any || act[i];
+            pend = pend || (!act[i] && st[i].xpend);
+          }
+          if (!any && pend) {
+            // the last iteration's x += alpha p, which a following forward pass would have applied
+            CK(launch_cg_flush<Tf>(d, p, c->d_st, 6 * c->g.M, n, c->stream));
+            for (int i = 0; i < n; ++i) st[i].xpend = 0;
+            CKS(write_states(c, st));
+          }
+        }
+      }
+      if (mixed && !fourier) {  // x += d, d = 0
         CK(launch_add_correction(reinterpret_cast<const float*>(d), x64, (long long)n * 6 * c->g.M, c->stream));
         CK(cudaMemsetAsync(d, 0, fb, c->stream));
       }
@@ -1222,7 +1406,7 @@ hom_status solve_system(hom_ctx* c, int n, const double* dE, const double* b64, 
         for (int i = 0; i < n; ++i) {
           if (!act[i]) continue;
           if (refine[i] > 0 || st[i].tol <= tol) tight[i] = 1, any_tight = true;
-          else loose[i] = 1, any_loose = true;
+          else if (!fourier) loose[i] = 1, any_loose = true;   // its d is compatible by construction
         }
         if (any_loose) {
           for (int i = 0; i < n; ++i) st[i].active = loose[i];
@@ -1711,8 +1895,15 @@ HOM_API int64_t hom_estimate_bytes(const int32_t grid[3], int32_t order, int32_t
   b += scratch(fp32 ? 8 : 16);
   if (fp32) b += scratch(16);
   const long long nl = loads_of_order(order), tf = fp32 ? 4 : 8;
-  b += 2 * nl * 6 * M * tf;                      // r, p
-  long long slot3 = fp32 ? nl * 6 * M * 4 : 0;   // FP32 correction d
+  // r, p and (FP32) the correction d: six real components, or in Fourier space three complex ones
+  Geo g{};
+  g.n2 = (int)n2;
+  g.n3 = (int)n3;
+  g.h = (int)(n1 / 2);
+  g.plane_c = plane_c;
+  const long long vec = fp32 ? nl * std::max(cg_vector_elems(g) * 8, 6 * M * 4) : nl * 6 * M * tf;
+  b += 2 * vec;
+  long long slot3 = fp32 ? vec : 0;
   if (order >= 1) {
     b += nl * 6 * M * 8;                         // right-hand sides
     slot3 = std::max(slot3, nl * 9 * M * 8);     // p and g of the right-hand-side build

@@ -55,12 +55,12 @@ struct RhsState {
   int sconv;         // 1: the half step s already met the tolerance (omega = 0, x += alpha p)
   int stall;         // 1: end the sweep when the residual stalls (FP32 sweeps of the refinement)
   int xpend;         // CG: x += alpha p of the last iteration is still to be applied (the next
-                     // forward pass applies it while it reads p; after a sweep, cg_flush does)
+                     // forward pass applies it while it reads p; after a sweep, cg_flush or cg_z_inv does)
 };
 
 // FWD_TAU: tau = (C - C0) : (in + E)     (polarization, Eq. auxiliary_problem)
 // FWD_STRESS: tau = C : (in + E)         (stress; -Gamma0 * sigma is the equilibrium residual)
-// FWD_CG: x += alpha p, p = r + beta p, tau = C : p   (CG: the previous iteration's update of x and
+// FWD_CG: x += alpha p, p = r + beta p, tau = C : p   (FP64 CG: the previous iteration's update of x and
 //         the new direction; A p = Gamma0 * (C : p) on compatible p)
 // FWD_COPY: tau = in                     (plain transform)
 // FWD_C0: tau = C0 : in                  (-Gamma0 * (C0 : in) is minus the compatible part of in)
@@ -70,7 +70,9 @@ enum FwdMode { FWD_TAU = 0, FWD_CG = 1, FWD_COPY = 2, FWD_STRESS = 3, FWD_C0 = 4
 // Z_DISP: forward z FFT of a strain, displacement u_hat (3 components), inverse z FFT
 // Z_RHS: forward z FFT of (p, g), -Gamma0_hat : (p_hat + theta_hat), inverse z FFT
 enum ZMode { Z_GAMMA = 0, Z_FWD = 1, Z_INV = 2, Z_DISP = 3, Z_RHS = 4, Z_GREEN = 5 };
-enum InvMode { INV_STORE = 0, INV_CG = 1 };
+// INV_STORE: out = out_scale eta (+ b - xsub); INV_CG: r += alpha eta; INV_ADD: out (FP64) += out_scale eta of
+// FP32 transforms (only the <double, float> kernels)
+enum InvMode { INV_STORE = 0, INV_CG = 1, INV_ADD = 2 };
 enum FinKind { FIN_NONE = 0, FIN_RHS = 1, FIN_BASIC = 2, FIN_CG = 3, FIN_RESID = 4, FIN_ENERGY = 5 };
 
 template <typename Tf, typename T>

@@ -14,6 +14,8 @@
 // k1..k5).  The polarization of component c therefore needs only component c, and
 // one CTA transforms one (rhs, component, z-plane) without touching the others.
 #pragma once
+#include <type_traits>
+
 #include "internal.h"
 
 namespace hom {
@@ -34,6 +36,10 @@ template <> struct PlaneCfg<double> {
 template <> struct PlaneCfg<df64> {
   static constexpr int kEPT = 16, kMaxThreads = 512, kMinBlocks = 1, kBatch = 4;
 };
+// CG on real fields (FWD_CG, INV_CG) runs in FP64 only: FP32 CG keeps its vectors in Fourier space
+template <typename T> constexpr bool kRealCg = std::is_same<T, double>::value;
+// FP32 transforms whose epilogue adds to an FP64 field (INV_ADD): a kernel of its own
+template <typename Tf, typename T> constexpr bool kInvAdds = sizeof(Tf) == 8 && sizeof(T) == 4;
 // threads of a plane CTA: every element of the n2 x h plane has a slot, whole warps, >= 128
 template <typename T>
 inline int plane_threads(const Geo& g) {
@@ -103,6 +109,10 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
 }
 
+// Prefetch of the 128-byte line of an address into L2.
+__device__ __forceinline__ void prefetch_line_l2(const void* ptr) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(ptr));
+}
 // Bulk prefetch of a contiguous global range into L2 (TMA, sm_90+).  bytes must be a multiple
 // of 16 and ptr 16-byte aligned; the range must lie inside one allocation.  Issued by one thread.
 __device__ __forceinline__ void prefetch_l2(const void* ptr, unsigned bytes) {
@@ -147,6 +157,49 @@ __device__ __forceinline__ bool publish_and_collect(double (&v)[NQ], double* par
     }
   }
   return last;
+}
+
+// The same for a reduction that one warp does alone (all 32 lanes call it): v is this CTA's totals in
+// lane 0.  Returns true in the warp of the CTA that drew the last ticket, with the grand totals in
+// lane 0; the CTA's other warps need not wait for it.
+template <int NQ>
+__device__ __forceinline__ bool warp_publish_and_collect(double (&v)[NQ], double* part, unsigned* cnt, int ncta, int cta) {
+  const int lane = threadIdx.x & 31;
+  unsigned t = 0;
+  if (lane == 0) {
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) part[q * ncta + cta] = v[q];
+    __threadfence();
+    t = atomicAdd(cnt, 1u);
+  }
+  if (__shfl_sync(0xffffffffu, t, 0) != (unsigned)(ncta - 1)) return false;
+  __threadfence();
+  double s[NQ];
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) s[q] = 0.0;
+  for (int i = lane; i < ncta; i += 32) {
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) s[q] += __ldcg(part + q * ncta + i);
+  }
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s[q] += __shfl_down_sync(0xffffffffu, s[q], o);
+    v[q] = s[q];
+  }
+  if (lane == 0) *cnt = 0u;
+  return true;
+}
+// Sums n values of shared memory in FP64 with one warp; the total is valid in lane 0.  (A warp sum per
+// warp of the CTA would cost as many FP64 instructions in each of them, on a pipe that takes 16
+// cycles per warp instruction here.)
+template <typename T>
+__device__ __forceinline__ double warp_sum_f64(const T* x, int n) {
+  double s = 0.0;
+  for (int i = threadIdx.x & 31; i < n; i += 32) s += (double)x[i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  return s;
 }
 
 __device__ __forceinline__ void finalize_state(int kind, RhsState& s, const double* v, double invM) {

@@ -6,11 +6,11 @@
 // columns [qCb, (q+1)Cb) of the half spectrum (Cb = (N1/2) / Q) for the y-axis work; between the
 // two the plane is transposed through distributed shared memory: each CTA reads its column block
 // out of the other CTAs' row blocks.  The forward pass applies the same prologues as plane_fwd
-// (polarization, Eq. auxiliary_problem; stress; CG direction; copy; C0) to its rows, runs the
+// (polarization, Eq. auxiliary_problem; stress; copy; C0) to its rows, runs the
 // packed real-to-complex row FFT, the transpose, the column FFT and writes its columns of the
 // spectrum; the inverse pass reads its columns, runs the inverse column FFT, the transpose, the
-// complex-to-real merge and row FFT, and the same epilogues as plane_inv (store, fixed-point step,
-// CG vector updates) with their FP64 reductions.
+// complex-to-real merge and row FFT, and the same epilogues as plane_inv (store, fixed-point step)
+// with their FP64 reductions.
 //
 // Compared with the split x and y passes, the intermediate half spectrum between the x and y
 // transforms never leaves the chip: two fewer spectrum sweeps through HBM per direction.
@@ -42,7 +42,6 @@ static size_t pc_smem_bytes(const Geo& g, size_t elem, size_t real) {
 
 template <typename Tf, typename T, int EPT>
 __global__ void __launch_bounds__(kPcMaxThreads, 1) plane_fwd_cluster_kernel(const FwdArgs<Tf, T> a) {
-  constexpr int kBatch = PlaneCfg<T>::kBatch;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cg::cluster_group cl = cg::this_cluster();
   const Geo& g = a.g;
@@ -58,9 +57,6 @@ __global__ void __launch_bounds__(kPcMaxThreads, 1) plane_fwd_cluster_kernel(con
   cx<T>* twy = twh + h;
   cx<T>* tw1 = twy + n2;
   T* tab = reinterpret_cast<T*>(tw1 + h + 1);
-  size_t off = align16((size_t)(R * P + n2 + h + n2 + h + 1) * sizeof(cx<T>) + 2 * 256 * sizeof(T));
-  double* sh = reinterpret_cast<double*>(smem_raw + off);
-  int* flag = reinterpret_cast<int*>(sh + 64);
   const int tid = threadIdx.x, nthr = blockDim.x;
 
   for (int i = tid; i < h; i += nthr) twh[i] = ldg_cx(a.tw_h + i);
@@ -81,8 +77,7 @@ __global__ void __launch_bounds__(kPcMaxThreads, 1) plane_fwd_cluster_kernel(con
   const long long foff = ((long long)(rhs * a.in_ncomp + c) * g.n3 + z) * plane_sz + (long long)y0 * n1;
   const long long blk_sz = (long long)R * n1;             // voxels of this CTA's rows
   if (a.prof != nullptr && tid == 0) {
-    long long fields = (a.mode == FWD_CG) ? (a.st[rhs].restart ? 2 : 5)
-                                          : ((a.mode == FWD_COPY || a.mode == FWD_C0 || a.in != nullptr) ? 1 : 0);
+    long long fields = (a.mode == FWD_COPY || a.mode == FWD_C0 || a.in != nullptr) ? 1 : 0;
     long long b = fields * blk_sz * (long long)sizeof(Tf) + (long long)n2 * Cb * (long long)sizeof(cx<T>);
     if (q == 0) b += (long long)n2 * (long long)sizeof(cx<T>);
     if (a.mode != FWD_COPY && a.mode != FWD_C0) b += blk_sz;
@@ -90,7 +85,6 @@ __global__ void __launch_bounds__(kPcMaxThreads, 1) plane_fwd_cluster_kernel(con
     atomicAdd(a.prof + 1, (unsigned long long)blk_sz);
   }
   const uint8_t* php = a.phase + (long long)rve * g.M + (long long)z * plane_sz + (long long)y0 * n1;
-  T acc = (T)0;
   const int total = R * h;   // complex elements of this CTA's rows (flat index e = row * h + col)
 
   if (a.mode == FWD_TAU || a.mode == FWD_STRESS) {
@@ -103,50 +97,6 @@ __global__ void __launch_bounds__(kPcMaxThreads, 1) plane_fwd_cluster_kernel(con
       if (a.in != nullptr) ld2<Tf>(a.in + foff + o, v0, v1);
       const uchar2 ph = *reinterpret_cast<const uchar2*>(php + o);
       buf[row * P + col] = mk<T>(w[ph.x] * ((T)v0 + ec), w[ph.y] * ((T)v1 + ec));
-    }
-  } else if (a.mode == FWD_CG) {
-    // the loads of kBatch elements per thread are issued before the first store of p
-    const RhsState& s = a.st[rhs];
-    const bool restart = (s.restart != 0);
-    const T beta = restart ? (T)0 : (T)s.beta;
-    const T alpha = restart ? (T)0 : (T)s.alpha;
-    const Tf* rp = a.r + foff;
-    Tf* pp = a.p + foff;
-    Tf* xp = a.x + foff;
-    for (int e0 = tid; e0 < total; e0 += kBatch * nthr) {
-      Tf r0[kBatch], r1[kBatch], p0[kBatch], p1[kBatch], x0[kBatch], x1[kBatch];
-      uchar2 ph[kBatch];
-      int rw[kBatch];
-#pragma unroll
-      for (int j = 0; j < kBatch; ++j) {
-        const int e = e0 + j * nthr;
-        rw[j] = (int)g.fd_h.div((unsigned)e);
-        p0[j] = 0;
-        p1[j] = 0;
-        if (e < total) {
-          const int o = rw[j] * n1 + 2 * (e - rw[j] * h);
-          ld2<Tf>(rp + o, r0[j], r1[j]);
-          if (!restart) {   // a restart neither reads the old p nor has an update of x pending
-            ld2<Tf>(pp + o, p0[j], p1[j]);
-            ld2<Tf>(xp + o, x0[j], x1[j]);
-          }
-          ph[j] = *reinterpret_cast<const uchar2*>(php + o);
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < kBatch; ++j) {
-        const int e = e0 + j * nthr;
-        if (e < total) {
-          const int col = e - rw[j] * h, o = rw[j] * n1 + 2 * col;
-          if (!restart) st2<Tf>(xp + o, (Tf)((T)x0[j] + alpha * (T)p0[j]), (Tf)((T)x1[j] + alpha * (T)p1[j]));
-          const T q0 = (T)r0[j] + beta * (T)p0[j];
-          const T q1 = (T)r1[j] + beta * (T)p1[j];
-          st2<Tf>(pp + o, (Tf)q0, (Tf)q1);
-          const T c0 = tab[a.n_phase + ph[j].x], c1 = tab[a.n_phase + ph[j].y];
-          acc += c0 * q0 * q0 + c1 * q1 * q1;
-          buf[rw[j] * P + col] = mk<T>(c0 * q0, c1 * q1);
-        }
-      }
     }
   } else {  // FWD_COPY, FWD_C0
     T ch, cd;
@@ -241,21 +191,10 @@ __global__ void __launch_bounds__(kPcMaxThreads, 1) plane_fwd_cluster_kernel(con
   }
   if (q == 0)
     for (int ky = tid; ky < n2; ky += nthr) Sp[(long long)n2 * h + ky] = nyq[ky];
-
-  if (a.mode == FWD_CG) {
-    double v[1] = {(double)acc};
-    block_sum_f64<1>(v, sh);
-    const int ncta = a.ncomp * g.n3 * Q;
-    if (publish_and_collect<1>(v, a.part + (long long)rhs * 2 * ncta, a.cnt + rhs, ncta, (c * g.n3 + z) * Q + q,
-                               sh, flag)) {
-      if (threadIdx.x == 0) finalize_state(FIN_ENERGY, a.st[rhs], v, 1.0 / (double)g.M);
-    }
-  }
 }
 
 template <typename Tf, typename T, int EPT>
 __global__ void __launch_bounds__(kPcMaxThreads, 1) plane_inv_cluster_kernel(const InvArgs<Tf, T> a) {
-  constexpr int kBatch = PlaneCfg<T>::kBatch;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cg::cluster_group cl = cg::this_cluster();
   const Geo& g = a.g;
@@ -292,7 +231,7 @@ __global__ void __launch_bounds__(kPcMaxThreads, 1) plane_inv_cluster_kernel(con
   const long long plane_sz = (long long)n2 * n1;
   const long long blk_sz = (long long)R * n1;
   if (a.prof != nullptr && tid == 0) {
-    long long fields = (a.mode == INV_CG) ? 2 : 1 + (a.fin == FIN_BASIC);
+    long long fields = 1 + (a.fin == FIN_BASIC);
     long long b = fields * blk_sz * (long long)sizeof(Tf) + (long long)n2 * Cb * (long long)sizeof(cx<T>);
     if (q == 0) b += (long long)n2 * (long long)sizeof(cx<T>);
     if (a.b != nullptr) b += blk_sz * (long long)sizeof(double);
@@ -365,7 +304,7 @@ __global__ void __launch_bounds__(kPcMaxThreads, 1) plane_inv_cluster_kernel(con
   // epilogue on this CTA's rows of the real plane: x[2n] = Re z[n], x[2n+1] = Im z[n]
   T q0 = 0, q1 = 0;
   const int total = R * h;
-  if (a.mode == INV_STORE) {
+  {
     const long long foff = ((long long)(rhs * a.out_ncomp + c) * g.n3 + z) * plane_sz + (long long)y0 * n1;
     const T cw = (c == 0) ? c0h : c0d;
     for (int e = tid; e < total; e += nthr) {
@@ -385,36 +324,6 @@ __global__ void __launch_bounds__(kPcMaxThreads, 1) plane_inv_cluster_kernel(con
       }
       q1 += v0 * v0 + v1 * v1;
       st2<Tf>(a.out + o, (Tf)v0, (Tf)v1);
-    }
-  } else {  // INV_CG: q = A p = Gamma0 * (C : p) = -eta, r -= alpha q (x += alpha p: next forward pass)
-    const long long foff = ((long long)(rhs * 6 + c) * g.n3 + z) * plane_sz + (long long)y0 * n1;
-    const T alpha = (T)a.st[rhs].alpha;
-    const T cw = (c == 0) ? c0h : c0d;
-    Tf* rp = a.r + foff;
-    for (int e0 = tid; e0 < total; e0 += kBatch * nthr) {
-      Tf r0[kBatch], r1[kBatch];
-      int rw[kBatch];
-#pragma unroll
-      for (int j = 0; j < kBatch; ++j) {
-        const int e = e0 + j * nthr;
-        rw[j] = (int)g.fd_h.div((unsigned)e);
-        if (e < total) {
-          const int o = rw[j] * n1 + 2 * (e - rw[j] * h);
-          ld2<Tf>(rp + o, r0[j], r1[j]);
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < kBatch; ++j) {
-        const int e = e0 + j * nthr;
-        if (e < total) {
-          const int col = e - rw[j] * h, o = rw[j] * n1 + 2 * col;
-          const cx<T> v = buf[rw[j] * P + col];
-          const T ra = (T)r0[j] + alpha * v.re, rb = (T)r1[j] + alpha * v.im;
-          st2<Tf>(rp + o, (Tf)ra, (Tf)rb);
-          q0 += cw * (ra * ra + rb * rb);
-          q1 += ra * ra + rb * rb;
-        }
-      }
     }
   }
 

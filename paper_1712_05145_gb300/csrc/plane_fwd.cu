@@ -85,49 +85,51 @@ plane_fwd_kernel(const FwdArgs<Tf, T> a) {
         pl[row * P + c2] = mk<T>(w[ph.x] * ((T)v0 + ec), w[ph.y] * ((T)v1 + ec));
       }
     }
-  } else if (a.mode == FWD_CG) {
-    // Flat element index e = row * h + col; the loads of kBatch elements per thread are issued
-    // before the first store of p (which the compiler must assume may alias r).
-    const RhsState& s = a.st[rhs];
-    const bool restart = (s.restart != 0);
-    const T beta = restart ? (T)0 : (T)s.beta;
-    const T alpha = restart ? (T)0 : (T)s.alpha;
-    const Tf* rp = a.r + foff;
-    Tf* pp = a.p + foff;
-    Tf* xp = a.x + foff;
-    const int total = n2 * h;
-    for (int e0 = tid; e0 < total; e0 += kBatch * nthr) {
-      Tf r0[kBatch], r1[kBatch], p0[kBatch], p1[kBatch], x0[kBatch], x1[kBatch];
-      uchar2 ph[kBatch];
-      int rw[kBatch];
-      #pragma unroll
-      for (int j = 0; j < kBatch; ++j) {
-        const int e = e0 + j * nthr;
-        rw[j] = (int)g.fd_h.div((unsigned)e);
-        p0[j] = 0;
-        p1[j] = 0;
-        if (e < total) {
-          const int o = rw[j] * n1 + 2 * (e - rw[j] * h);
-          ld2<Tf>(rp + o, r0[j], r1[j]);
-          if (!restart) {   // a restart neither reads the old p nor has an update of x pending
-            ld2<Tf>(pp + o, p0[j], p1[j]);
-            ld2<Tf>(xp + o, x0[j], x1[j]);
+  } else if (kRealCg<T> && a.mode == FWD_CG) {
+    if constexpr (kRealCg<T>) {
+      // Flat element index e = row * h + col; the loads of kBatch elements per thread are issued
+      // before the first store of p (which the compiler must assume may alias r).
+      const RhsState& s = a.st[rhs];
+      const bool restart = (s.restart != 0);
+      const T beta = restart ? (T)0 : (T)s.beta;
+      const T alpha = restart ? (T)0 : (T)s.alpha;
+      const Tf* rp = a.r + foff;
+      Tf* pp = a.p + foff;
+      Tf* xp = a.x + foff;
+      const int total = n2 * h;
+      for (int e0 = tid; e0 < total; e0 += kBatch * nthr) {
+        Tf r0[kBatch], r1[kBatch], p0[kBatch], p1[kBatch], x0[kBatch], x1[kBatch];
+        uchar2 ph[kBatch];
+        int rw[kBatch];
+        #pragma unroll
+        for (int j = 0; j < kBatch; ++j) {
+          const int e = e0 + j * nthr;
+          rw[j] = (int)g.fd_h.div((unsigned)e);
+          p0[j] = 0;
+          p1[j] = 0;
+          if (e < total) {
+            const int o = rw[j] * n1 + 2 * (e - rw[j] * h);
+            ld2<Tf>(rp + o, r0[j], r1[j]);
+            if (!restart) {   // a restart neither reads the old p nor has an update of x pending
+              ld2<Tf>(pp + o, p0[j], p1[j]);
+              ld2<Tf>(xp + o, x0[j], x1[j]);
+            }
+            ph[j] = *reinterpret_cast<const uchar2*>(php + o);
           }
-          ph[j] = *reinterpret_cast<const uchar2*>(php + o);
         }
-      }
-      #pragma unroll
-      for (int j = 0; j < kBatch; ++j) {
-        const int e = e0 + j * nthr;
-        if (e < total) {
-          const int col = e - rw[j] * h, o = rw[j] * n1 + 2 * col;
-          if (!restart) st2<Tf>(xp + o, (Tf)((T)x0[j] + alpha * (T)p0[j]), (Tf)((T)x1[j] + alpha * (T)p1[j]));
-          const T q0 = (T)r0[j] + beta * (T)p0[j];
-          const T q1 = (T)r1[j] + beta * (T)p1[j];
-          st2<Tf>(pp + o, (Tf)q0, (Tf)q1);
-          const T c0 = tab[a.n_phase + ph[j].x], c1 = tab[a.n_phase + ph[j].y];
-          acc += c0 * q0 * q0 + c1 * q1 * q1;
-          pl[rw[j] * P + col] = mk<T>(c0 * q0, c1 * q1);
+        #pragma unroll
+        for (int j = 0; j < kBatch; ++j) {
+          const int e = e0 + j * nthr;
+          if (e < total) {
+            const int col = e - rw[j] * h, o = rw[j] * n1 + 2 * col;
+            if (!restart) st2<Tf>(xp + o, (Tf)((T)x0[j] + alpha * (T)p0[j]), (Tf)((T)x1[j] + alpha * (T)p1[j]));
+            const T q0 = (T)r0[j] + beta * (T)p0[j];
+            const T q1 = (T)r1[j] + beta * (T)p1[j];
+            st2<Tf>(pp + o, (Tf)q0, (Tf)q1);
+            const T c0 = tab[a.n_phase + ph[j].x], c1 = tab[a.n_phase + ph[j].y];
+            acc += c0 * q0 * q0 + c1 * q1 * q1;
+            pl[rw[j] * P + col] = mk<T>(c0 * q0, c1 * q1);
+          }
         }
       }
     }
@@ -209,7 +211,7 @@ plane_fwd_kernel(const FwdArgs<Tf, T> a) {
   }
   for (int ky = tid; ky < n2; ky += nthr) Sp[(long long)n2 * h + ky] = nyq[ky];
 
-  if (a.mode == FWD_CG) {
+  if (kRealCg<T> && a.mode == FWD_CG) {
     double v[1] = {(double)acc};
     block_sum_f64<1>(v, sh);
     const int ncta = a.ncomp * g.n3;

@@ -105,7 +105,19 @@ plane_inv_kernel(const InvArgs<Tf, T> a) {
   // epilogue on the real plane: x[2n] = Re z[n], x[2n+1] = Im z[n]
   const long long plane_sz = (long long)n2 * n1;
   T q0 = 0, q1 = 0;
-  if (a.mode == INV_STORE) {
+  if constexpr (kInvAdds<Tf, T>) {   // out += eta: an FP32 correction added to the FP64 field
+    const long long foff = ((long long)(rhs * a.out_ncomp + c) * g.n3 + z) * plane_sz;
+    #pragma unroll 4
+    for (int row = warp; row < n2; row += nwarp) {
+      for (int c2 = lane; c2 < h; c2 += 32) {
+        Tf* o = a.out + foff + (long long)row * n1 + 2 * c2;
+        const cx<T> e = pl[row * P + c2];
+        Tf o0, o1;
+        ld2<Tf>(o, o0, o1);
+        st2<Tf>(o, o0 + (Tf)(a.out_scale * e.re), o1 + (Tf)(a.out_scale * e.im));
+      }
+    }
+  } else if (a.mode == INV_STORE) {
     const long long foff = ((long long)(rhs * a.out_ncomp + c) * g.n3 + z) * plane_sz;
     const T cw = (c == 0) ? c0h : c0d;
     #pragma unroll 4
@@ -128,7 +140,7 @@ plane_inv_kernel(const InvArgs<Tf, T> a) {
         st2<Tf>(a.out + o, (Tf)v0, (Tf)v1);
       }
     }
-  } else {  // INV_CG: q = A p = Gamma0 * (C : p) = -eta, r -= alpha q (x += alpha p: next forward pass)
+  } else if constexpr (kRealCg<T>) {  // INV_CG: q = A p = Gamma0 * (C : p) = -eta, r -= alpha q (x += alpha p: next forward pass)
     // Flat element index e = row * h + col; each thread issues the loads of kBatch elements
     // before the first store, so that they are in flight together (a store to r may alias the
     // next load for the compiler, which would otherwise serialise load -> store chains).
@@ -192,6 +204,7 @@ cudaError_t launch_plane_inv(const InvArgs<Tf, T>& a, int nrhs, cudaStream_t s) 
 
 template cudaError_t launch_plane_inv<float, float>(const InvArgs<float, float>&, int, cudaStream_t);
 template cudaError_t launch_plane_inv<double, double>(const InvArgs<double, double>&, int, cudaStream_t);
+template cudaError_t launch_plane_inv<double, float>(const InvArgs<double, float>&, int, cudaStream_t);
 template cudaError_t launch_plane_inv<float, double>(const InvArgs<float, double>&, int, cudaStream_t);
 template cudaError_t launch_plane_inv<float, df64>(const InvArgs<float, df64>&, int, cudaStream_t);
 template cudaError_t launch_plane_inv<double, df64>(const InvArgs<double, df64>&, int, cudaStream_t);

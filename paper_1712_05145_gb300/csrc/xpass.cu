@@ -9,9 +9,7 @@
 
 namespace hom {
 
-// FP32 forward x pass: at most 64 registers, so four 256-thread CTAs fit an SM (74 registers and
-// three CTAs without the bound); the extra resident warps hide its field loads (512^3: 3.65 ->
-// 3.39 ms per launch), without spills.  The FP64 and double-float forms: at most 128 registers,
+// FP32 forward x pass: at most 64 registers, so four 256-thread CTAs fit an SM.  The FP64 and double-float forms: at most 128 registers,
 // two CTAs per SM (with a bound of one CTA the double-float form takes 156 registers and runs 30 %
 // slower).
 template <typename T> struct XfCfg { static constexpr int kMinBlocks = 2; };
@@ -89,52 +87,54 @@ __global__ void __launch_bounds__(256, XfCfg<T>::kMinBlocks) xpass_fwd_kernel(co
   c0_weights<T>(a.c0, rve, a.c0h, a.c0d, ch, cd);
   const T wc = (a.mode == FWD_C0) ? (c == 0 ? ch : cd) : (T)1;
 
-  if (a.mode == FWD_CG) {
-    // Flat index e = row * h + col over this block's rows (contiguous in the field); the loads of
-    // kBatch elements per thread are issued before the first store of p, which the compiler must
-    // assume may alias r, so that they are in flight together.
-    constexpr int kBatch = PlaneCfg<T>::kBatch;
-    const Tf* rp = a.r + cbase + r0 * n1;
-    Tf* pp = a.p + cbase + r0 * n1;
-    Tf* xp = a.x + cbase + r0 * n1;
-    const uint8_t* php = phase + r0 * n1;
-    const int total = nr * h;
-    for (int e0 = tid; e0 < rb * h; e0 += kBatch * nthr) {
-      Tf q0r[kBatch], q1r[kBatch], p0[kBatch], p1[kBatch], x0[kBatch], x1[kBatch];
-      uchar2 ph[kBatch];
-      int rw[kBatch];
+  if (kRealCg<T> && a.mode == FWD_CG) {
+    if constexpr (kRealCg<T>) {
+      // Flat index e = row * h + col over this block's rows (contiguous in the field); the loads of
+      // kBatch elements per thread are issued before the first store of p, which the compiler must
+      // assume may alias r, so that they are in flight together.
+      constexpr int kBatch = PlaneCfg<T>::kBatch;
+      const Tf* rp = a.r + cbase + r0 * n1;
+      Tf* pp = a.p + cbase + r0 * n1;
+      Tf* xp = a.x + cbase + r0 * n1;
+      const uint8_t* php = phase + r0 * n1;
+      const int total = nr * h;
+      for (int e0 = tid; e0 < rb * h; e0 += kBatch * nthr) {
+        Tf q0r[kBatch], q1r[kBatch], p0[kBatch], p1[kBatch], x0[kBatch], x1[kBatch];
+        uchar2 ph[kBatch];
+        int rw[kBatch];
 #pragma unroll
-      for (int j = 0; j < kBatch; ++j) {
-        const int e = e0 + j * nthr;
-        rw[j] = (int)g.fd_h.div((unsigned)e);
-        p0[j] = 0;
-        p1[j] = 0;
-        if (e < total) {
-          const int o = rw[j] * n1 + 2 * (e - rw[j] * h);
-          ld2<Tf>(rp + o, q0r[j], q1r[j]);
-          if (!restart) {   // a restart neither reads the old p nor has an update of x pending
-            ld2<Tf>(pp + o, p0[j], p1[j]);
-            ld2<Tf>(xp + o, x0[j], x1[j]);
+        for (int j = 0; j < kBatch; ++j) {
+          const int e = e0 + j * nthr;
+          rw[j] = (int)g.fd_h.div((unsigned)e);
+          p0[j] = 0;
+          p1[j] = 0;
+          if (e < total) {
+            const int o = rw[j] * n1 + 2 * (e - rw[j] * h);
+            ld2<Tf>(rp + o, q0r[j], q1r[j]);
+            if (!restart) {   // a restart neither reads the old p nor has an update of x pending
+              ld2<Tf>(pp + o, p0[j], p1[j]);
+              ld2<Tf>(xp + o, x0[j], x1[j]);
+            }
+            ph[j] = *reinterpret_cast<const uchar2*>(php + o);
           }
-          ph[j] = *reinterpret_cast<const uchar2*>(php + o);
         }
-      }
 #pragma unroll
-      for (int j = 0; j < kBatch; ++j) {
-        const int e = e0 + j * nthr;
-        if (e >= rb * h) continue;
-        const int col = e - rw[j] * h;
-        cx<T> val = mk<T>(0, 0);
-        if (e < total) {
-          const int o = rw[j] * n1 + 2 * col;
-          if (!restart) st2<Tf>(xp + o, (Tf)((T)x0[j] + alpha * (T)p0[j]), (Tf)((T)x1[j] + alpha * (T)p1[j]));
-          const T q0 = (T)q0r[j] + beta * (T)p0[j], q1 = (T)q1r[j] + beta * (T)p1[j];
-          st2<Tf>(pp + o, (Tf)q0, (Tf)q1);
-          const T c0 = tab[a.n_phase + ph[j].x], c1 = tab[a.n_phase + ph[j].y];
-          acc += c0 * q0 * q0 + c1 * q1 * q1;
-          val = mk<T>(c0 * q0, c1 * q1);
+        for (int j = 0; j < kBatch; ++j) {
+          const int e = e0 + j * nthr;
+          if (e >= rb * h) continue;
+          const int col = e - rw[j] * h;
+          cx<T> val = mk<T>(0, 0);
+          if (e < total) {
+            const int o = rw[j] * n1 + 2 * col;
+            if (!restart) st2<Tf>(xp + o, (Tf)((T)x0[j] + alpha * (T)p0[j]), (Tf)((T)x1[j] + alpha * (T)p1[j]));
+            const T q0 = (T)q0r[j] + beta * (T)p0[j], q1 = (T)q1r[j] + beta * (T)p1[j];
+            st2<Tf>(pp + o, (Tf)q0, (Tf)q1);
+            const T c0 = tab[a.n_phase + ph[j].x], c1 = tab[a.n_phase + ph[j].y];
+            acc += c0 * q0 * q0 + c1 * q1 * q1;
+            val = mk<T>(c0 * q0, c1 * q1);
+          }
+          pl[rw[j] * P + col] = val;
         }
-        pl[rw[j] * P + col] = val;
       }
     }
   } else {
@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(256, XfCfg<T>::kMinBlocks) xpass_fwd_kernel(co
     for (int col = lane; col < h; col += 32) dst[col] = pl[lr * P + col];
   }
 
-  if (a.mode == FWD_CG) {
+  if (kRealCg<T> && a.mode == FWD_CG) {
     double v[1] = {(double)acc};
     block_sum_f64<1>(v, sh);
     const int ncta = a.ncomp * g.nrb;
@@ -297,7 +297,19 @@ __global__ void __launch_bounds__(256) xpass_inv_kernel(const InvArgs<Tf, T> a) 
   T ch, cd;
   c0_weights<T>(a.c0, rve_of(rhs, a.rve_loads), a.c0h, a.c0d, ch, cd);
   const T cw = (c == 0) ? ch : cd;
-  if (a.mode == INV_STORE) {
+  if constexpr (kInvAdds<Tf, T>) {   // out += eta: an FP32 correction added to the FP64 field
+    const long long cbase = (long long)(rhs * a.out_ncomp + c) * g.M;
+#pragma unroll 4
+    for (int lr = warp; lr < nr; lr += nwarp) {
+      for (int c2 = lane; c2 < h; c2 += 32) {
+        Tf* o = a.out + cbase + (r0 + lr) * n1 + 2 * c2;
+        const cx<T> e = pl[lr * P + c2];
+        Tf o0, o1;
+        ld2<Tf>(o, o0, o1);
+        st2<Tf>(o, o0 + (Tf)(a.out_scale * e.re), o1 + (Tf)(a.out_scale * e.im));
+      }
+    }
+  } else if (a.mode == INV_STORE) {
     const long long cbase = (long long)(rhs * a.out_ncomp + c) * g.M;
 #pragma unroll 4
     for (int lr = warp; lr < nr; lr += nwarp) {
@@ -319,7 +331,7 @@ __global__ void __launch_bounds__(256) xpass_inv_kernel(const InvArgs<Tf, T> a) 
         st2<Tf>(a.out + o, (Tf)v0, (Tf)v1);
       }
     }
-  } else {  // INV_CG: r -= alpha A p with A p = -eta (x += alpha p: next forward pass)
+  } else if constexpr (kRealCg<T>) {  // INV_CG: r -= alpha A p with A p = -eta (x += alpha p: next forward pass)
     // flat index e = row * h + col; kBatch elements' loads in flight before the first store
     constexpr int kBatch = PlaneCfg<T>::kBatch;
     const long long cbase = (long long)(rhs * 6 + c) * g.M + r0 * n1;
@@ -400,6 +412,7 @@ template cudaError_t launch_xpass_fwd<float, float>(const FwdArgs<float, float>&
 template cudaError_t launch_xpass_fwd<double, double>(const FwdArgs<double, double>&, int, cudaStream_t);
 template cudaError_t launch_xpass_inv<float, float>(const InvArgs<float, float>&, int, cudaStream_t);
 template cudaError_t launch_xpass_inv<double, double>(const InvArgs<double, double>&, int, cudaStream_t);
+template cudaError_t launch_xpass_inv<double, float>(const InvArgs<double, float>&, int, cudaStream_t);
 template cudaError_t launch_xpass_inv<float, double>(const InvArgs<float, double>&, int, cudaStream_t);
 template cudaError_t launch_xpass_fwd<double, df64>(const FwdArgs<double, df64>&, int, cudaStream_t);
 template cudaError_t launch_xpass_inv<float, df64>(const InvArgs<float, df64>&, int, cudaStream_t);
