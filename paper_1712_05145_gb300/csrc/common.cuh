@@ -10,6 +10,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 namespace hom {
 
 // Double-float number: the unevaluated sum hi + lo of two floats (|lo| <= ulp(hi) / 2), about
@@ -354,6 +356,32 @@ __device__ __forceinline__ void fft_pencils(cx<T>* buf, const Addr& addr, int n,
                                             const cx<T>* tw) {
 #define HOM_SEQ(NN, ...) \
   case NN: StageSeq<T, DIR, EPT, NN, 1, __VA_ARGS__>::run(buf, addr, npen, npd, tw); break;
+  if constexpr (std::is_same<T, df64>::value) {
+    // a double-float butterfly keeps 4 registers per value, and its sums are long dependent chains: radices
+    // up to 8 let twice the warps be resident
+    switch (n) {
+      case 1: break;
+      HOM_SEQ(2, 2)
+      HOM_SEQ(3, 3)
+      HOM_SEQ(4, 4)
+      HOM_SEQ(6, 3, 2)
+      HOM_SEQ(8, 8)
+      HOM_SEQ(12, 4, 3)
+      HOM_SEQ(16, 4, 4)
+      HOM_SEQ(24, 8, 3)
+      HOM_SEQ(32, 8, 4)
+      HOM_SEQ(48, 4, 4, 3)
+      HOM_SEQ(64, 8, 8)
+      HOM_SEQ(96, 8, 4, 3)
+      HOM_SEQ(128, 8, 4, 4)
+      HOM_SEQ(192, 8, 8, 3)
+      HOM_SEQ(256, 8, 8, 4)
+      HOM_SEQ(384, 8, 4, 4, 3)
+      HOM_SEQ(512, 8, 8, 8)
+      default: break;
+    }
+    return;
+  }
   switch (n) {
     case 1: break;  // a single plane along z (two-dimensional cells): the identity
     HOM_SEQ(2, 2)

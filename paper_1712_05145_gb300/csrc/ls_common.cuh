@@ -21,6 +21,9 @@
 namespace hom {
 
 constexpr int kEPT = 16;
+// elements per thread of a transform type: the double-float transforms take twice the threads
+template <typename T> constexpr int kEptOf = kEPT;
+template <> inline constexpr int kEptOf<df64> = 8;
 // Launch shape of the plane kernels per compute precision: 16 elements per thread, CTAs of up
 // to 512 threads.  (8 elements per thread with 1024-thread CTAs and 32 registers, which doubles
 // the resident warps, measured slower at 128^3: the extra radix stage and register spills cost
@@ -33,8 +36,10 @@ template <> struct PlaneCfg<float> {   // 64 registers: 2 CTAs per SM
 template <> struct PlaneCfg<double> {
   static constexpr int kEPT = 16, kMaxThreads = 512, kMinBlocks = 1, kBatch = 4;
 };
+// 1024 threads at 64 registers (radices up to 8, see fft_pencils): a 128^2 plane fills an SM's shared
+// memory, and 16 resident warps hid too little of the double-float sums' latency
 template <> struct PlaneCfg<df64> {
-  static constexpr int kEPT = 16, kMaxThreads = 512, kMinBlocks = 1, kBatch = 4;
+  static constexpr int kEPT = 8, kMaxThreads = 1024, kMinBlocks = 1, kBatch = 2;
 };
 // CG on real fields (FWD_CG, INV_CG) runs in FP64 only: FP32 CG keeps its vectors in Fourier space
 template <typename T> constexpr bool kRealCg = std::is_same<T, double>::value;

@@ -9,14 +9,13 @@
 
 namespace hom {
 
-// FP32 forward x pass: at most 64 registers, so four 256-thread CTAs fit an SM.  The FP64 and double-float forms: at most 128 registers,
-// two CTAs per SM (with a bound of one CTA the double-float form takes 156 registers and runs 30 %
-// slower).
+// FP32 forward x pass: at most 64 registers, so four 256-thread CTAs fit an SM.  The FP64 form: at
+// most 128 registers, two CTAs per SM.  The double-float form: two CTAs of 512 threads (64 registers).
 template <typename T> struct XfCfg { static constexpr int kMinBlocks = 2; };
 template <> struct XfCfg<float> { static constexpr int kMinBlocks = 4; };
 
 template <typename Tf, typename T, int EPT>
-__global__ void __launch_bounds__(256, XfCfg<T>::kMinBlocks) xpass_fwd_kernel(const FwdArgs<Tf, T> a) {
+__global__ void __launch_bounds__(256 * (kEPT / EPT), XfCfg<T>::kMinBlocks) xpass_fwd_kernel(const FwdArgs<Tf, T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const Geo& g = a.g;
   const int blk = blockIdx.x, c = blockIdx.y, lrhs = blockIdx.z, rhs = a.rhs0 + lrhs;
@@ -211,7 +210,7 @@ __global__ void __launch_bounds__(256, XfCfg<T>::kMinBlocks) xpass_fwd_kernel(co
 }
 
 template <typename Tf, typename T, int EPT>
-__global__ void __launch_bounds__(256) xpass_inv_kernel(const InvArgs<Tf, T> a) {
+__global__ void __launch_bounds__(256 * (kEPT / EPT), std::is_same<T, df64>::value ? 2 : 1) xpass_inv_kernel(const InvArgs<Tf, T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const Geo& g = a.g;
   const int blk = blockIdx.x, c = blockIdx.y, lrhs = blockIdx.z, rhs = a.rhs0 + lrhs;
@@ -386,12 +385,12 @@ cudaError_t launch_xpass_fwd(const FwdArgs<Tf, T>& a, int nrhs, cudaStream_t s) 
   if ((long long)a.g.rb * a.g.h > (long long)kEPT * a.g.thr_x || a.g.thr_x > 256 || a.n_phase > 256)
     return cudaErrorInvalidValue;
   const size_t smem = xpass_smem_bytes(a.g, sizeof(cx<T>));
-  auto k = xpass_fwd_kernel<Tf, T, kEPT>;
+  auto k = xpass_fwd_kernel<Tf, T, kEptOf<T>>;
   cudaError_t e = set_smem(k, smem);
   if (e != cudaSuccess) return e;
   dim3 grid(a.g.nrb, a.ncomp, nrhs);
   count_launch();
-  k<<<grid, a.g.thr_x, smem, s>>>(a);
+  k<<<grid, a.g.thr_x * (kEPT / kEptOf<T>), smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -399,12 +398,12 @@ template <typename Tf, typename T>
 cudaError_t launch_xpass_inv(const InvArgs<Tf, T>& a, int nrhs, cudaStream_t s) {
   if ((long long)a.g.rb * a.g.h > (long long)kEPT * a.g.thr_x || a.g.thr_x > 256) return cudaErrorInvalidValue;
   const size_t smem = xpass_smem_bytes(a.g, sizeof(cx<T>));
-  auto k = xpass_inv_kernel<Tf, T, kEPT>;
+  auto k = xpass_inv_kernel<Tf, T, kEptOf<T>>;
   cudaError_t e = set_smem(k, smem);
   if (e != cudaSuccess) return e;
   dim3 grid(a.g.nrb, a.ncomp, nrhs);
   count_launch();
-  k<<<grid, a.g.thr_x, smem, s>>>(a);
+  k<<<grid, a.g.thr_x * (kEPT / kEptOf<T>), smem, s>>>(a);
   return cudaGetLastError();
 }
 

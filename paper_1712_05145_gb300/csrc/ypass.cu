@@ -37,7 +37,7 @@ __device__ __forceinline__ void y_separate(cx<T>* buf, int pitch, cx<T>* nyq, in
 }
 
 template <typename T, int DIR, int EPT>
-__global__ void __launch_bounds__(512) ypass_kernel(const cx<T>* __restrict__ tw_n2, cx<T>* S, const Geo g,
+__global__ void __launch_bounds__(512 * (kEPT / EPT)) ypass_kernel(const cx<T>* __restrict__ tw_n2, cx<T>* S, const Geo g,
                                                     int ncomp, int s_ncomp, unsigned long long* prof,
                                                     const RhsState* st, int rhs0) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -89,17 +89,17 @@ cudaError_t launch_ypass(const cx<T>* tw_n2, cx<T>* S, const Geo& g, int ncomp, 
   const size_t smem = (size_t)(g.n2 * TY + g.n2) * sizeof(cx<T>);
   dim3 grid(g.h / TY, g.n3, ncomp * nrhs);
   if (dir < 0) {
-    auto k = ypass_kernel<T, -1, kEPT>;
+    auto k = ypass_kernel<T, -1, kEptOf<T>>;
     cudaError_t e = set_smem(k, smem);
     if (e != cudaSuccess) return e;
     count_launch();
-    k<<<grid, g.thr_y, smem, s>>>(tw_n2, S, g, ncomp, s_ncomp, prof, st, rhs0);
+    k<<<grid, g.thr_y * (kEPT / kEptOf<T>), smem, s>>>(tw_n2, S, g, ncomp, s_ncomp, prof, st, rhs0);
   } else {
-    auto k = ypass_kernel<T, +1, kEPT>;
+    auto k = ypass_kernel<T, +1, kEptOf<T>>;
     cudaError_t e = set_smem(k, smem);
     if (e != cudaSuccess) return e;
     count_launch();
-    k<<<grid, g.thr_y, smem, s>>>(tw_n2, S, g, ncomp, s_ncomp, prof, st, rhs0);
+    k<<<grid, g.thr_y * (kEPT / kEptOf<T>), smem, s>>>(tw_n2, S, g, ncomp, s_ncomp, prof, st, rhs0);
   }
   return cudaGetLastError();
 }

@@ -26,9 +26,10 @@ namespace hom {
 constexpr int kZcComps = 6;            // CTAs per cluster: one per Kelvin component
 constexpr int kZcMaxElems = kEPT * 512;
 constexpr size_t kZcMaxSmem = 80 * 1024;
-// two 512-thread CTAs per SM in FP32 (64 registers); the 16-byte types keep more registers
-template <typename T> struct ZcCfg { static constexpr int kMinBlocks = 1; };
-template <> struct ZcCfg<float> { static constexpr int kMinBlocks = 2; };
+// two 512-thread CTAs per SM in FP32 (64 registers), one of 1024 threads in double-float; FP64 keeps
+// more registers
+template <typename T> struct ZcCfg { static constexpr int kMinBlocks = 1, kThreads = 512 * (kEPT / kEptOf<T>); };
+template <> struct ZcCfg<float> { static constexpr int kMinBlocks = 2, kThreads = 512; };
 
 // -Gamma0_hat(xi) : tau_hat at tile element q (column f0 + q mod 2^lg, z-plane q / 2^lg), in place on
 // its six Kelvin components k; columns past the plane are left as they are
@@ -51,7 +52,7 @@ __device__ __forceinline__ void contract_point(const Geo& g, const ZArgs<T>& a, 
 }
 
 template <typename T, int EPT>
-__global__ void __cluster_dims__(kZcComps, 1, 1) __launch_bounds__(512, ZcCfg<T>::kMinBlocks) zcluster_kernel(const ZArgs<T> a) {
+__global__ void __cluster_dims__(kZcComps, 1, 1) __launch_bounds__(ZcCfg<T>::kThreads, ZcCfg<T>::kMinBlocks) zcluster_kernel(const ZArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cg::cluster_group cl = cg::this_cluster();
   const Geo& g = a.g;
@@ -223,7 +224,7 @@ bool zcluster_tiling(ZArgs<T>& a, int force_lg) {
   const long long tc = 1LL << best;
   a.ntiles = (int)((a.g.plane_c + tc - 1) / tc);
   const long long e = (long long)a.g.n3 * tc;
-  int thr = (int)((e + kEPT - 1) / kEPT);
+  int thr = (int)((e + kEptOf<T> - 1) / kEptOf<T>);
   thr = ((thr + 31) / 32) * 32;
   a.nthr = thr < 64 ? 64 : thr;
   a.fd_in = make_fastdiv((unsigned)tc);
@@ -237,10 +238,10 @@ template <typename T>
 cudaError_t launch_zcluster(const ZArgs<T>& a, int nrhs, cudaStream_t s) {
   const long long e = (long long)a.g.n3 * (1LL << a.tc_log2);
   if (a.mode != Z_GAMMA || a.ncomp_in != 6 || a.ncomp_out != 6 || !zcluster_tile_fits(a.g, sizeof(cx<T>), a.tc_log2) ||
-      e > (long long)kEPT * a.nthr || a.nthr > 512 || nrhs < 1 || (long long)a.ntiles * kZcComps > 0x7fffffffLL)
+      e > (long long)kEptOf<T> * a.nthr || a.nthr > ZcCfg<T>::kThreads || nrhs < 1 || (long long)a.ntiles * kZcComps > 0x7fffffffLL)
     return cudaErrorInvalidValue;
   const size_t smem = zcluster_smem(a.g, sizeof(cx<T>), a.tc_log2);
-  auto k = zcluster_kernel<T, kEPT>;
+  auto k = zcluster_kernel<T, kEptOf<T>>;
   cudaError_t err = set_smem(k, smem);
   if (err != cudaSuccess) return err;
   dim3 grid((unsigned)(a.ntiles * kZcComps), (unsigned)nrhs);
