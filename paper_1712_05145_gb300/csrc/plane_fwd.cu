@@ -265,7 +265,9 @@ size_t zpass_smem_bytes(const Geo& g, size_t elem, int ncomp, int tc_log2) {
   return ((size_t)ncomp * cstride + g.n3) * elem;
 }
 
-// z-pass tile: 2^lg consecutive spectrum columns (lg <= 4) whose pencils fit kEPT elements per
+// z-pass tile: 2^lg consecutive spectrum columns (lg <= 4; up to 8 on grids shallower than 16 planes, where 16
+// columns are too little work for a CTA: a two-dimensional cell's contraction kept 16 of 128 threads busy,
+// 0.22 ms at 512^2 in FP64, two loads) whose pencils fit kEPT elements per
 // thread at <= 512 threads and <= 64 KB of shared memory.  Among the tiles whose row reads cover
 // at least one 32-byte sector, the one with the most resident warps per SM wins (ties: the
 // wider tile); at 128^3 in FP32 that is 4 columns (192 threads, 5 CTAs per SM) rather than 8
@@ -278,7 +280,7 @@ static int zpass_threads(int ncomp, int n3, int lg) {
 }
 
 bool zpass_tile_fits(const Geo& g, size_t elem, int ncomp, int lg) {
-  return lg >= 0 && lg <= 4 && (size_t)ncomp * g.n3 * ((size_t)1 << lg) <= (size_t)kEPT * 512 &&
+  return lg >= 0 && lg <= (g.n3 < 16 ? 8 : 4) && (size_t)ncomp * g.n3 * ((size_t)1 << lg) <= (size_t)kEPT * 512 &&
          zpass_smem_bytes(g, elem, ncomp, lg) <= 64 * 1024;
 }
 
@@ -289,7 +291,7 @@ void zpass_tiling(ZArgs<T>& a, int force_lg) {
   long long best_warps = -1;
   const bool forced = force_lg >= 0 && zpass_tile_fits(a.g, elem, a.ncomp_in, force_lg);
   if (forced) best_lg = force_lg;
-  for (int lg = 4; lg >= 0 && !forced; --lg) {
+  for (int lg = 8; lg >= 0 && !forced; --lg) {
     if (!zpass_tile_fits(a.g, elem, a.ncomp_in, lg)) continue;
     if (best_lg >= 0 && ((size_t)1 << lg) * elem < 32) break;   // narrower than a sector
     const int thr = zpass_threads(a.ncomp_in, a.g.n3, lg);
