@@ -347,10 +347,10 @@ __global__ void __launch_bounds__(ZLaunch<N, TC>::threads, ZLaunch<N, TC>::min_b
     tw[i] = ldg_cx(a.tw_n3 + i);
     zt[i] = z_factors(g, a.green, a.gtab, i);
   }
-  // v = Gamma0_hat(q) : tau_hat from w = tau_hat q (STEP), or the components of a compatible strain (INIT)
+  // v = Gamma0_hat(q) : tau_hat from w = tau_hat q (STEP, RHS), or the components of a compatible strain (INIT)
   float c1 = 1.0f, c2h = 0.5f;
   const int rve = rve_of(rhs, a.rve_loads);
-  if (MODE == CGF_STEP) green_consts<float>(a.c0, rve, a.lam0, a.mu0, c1, c2h);
+  if (MODE != CGF_INIT) green_consts<float>(a.c0, rve, a.lam0, a.mu0, c1, c2h);
   c1 *= a.scale;
   c2h *= a.scale;
   const float alpha = MODE == CGF_STEP ? (float)a.st[rhs].alpha : 0.0f;
@@ -403,18 +403,22 @@ __global__ void __launch_bounds__(ZLaunch<N, TC>::threads, ZLaunch<N, TC>::min_b
         v1 = fma_cx(v1, -alpha, rl[o]);
         v2 = fma_cx(v2, -alpha, rl[o + comp_v]);
         v3 = fma_cx(v3, -alpha, rl[o + 2 * comp_v]);
+      } else if (MODE == CGF_RHS) {
+        v1 = v1 * -1.0f;
+        v2 = v2 * -1.0f;
+        v3 = v3 * -1.0f;
       }
       rl[o] = v1;
       rl[o + comp_v] = v2;
       rl[o + 2 * comp_v] = v3;
-      if (MODE == CGF_STEP) {
+      if (MODE != CGF_INIT) {
         const cx<float> d = fma_cx(v3, q3, fma_cx(v2, q2, v1 * q1));
         const float m = v1.re * v1.re + v1.im * v1.im + v2.re * v2.re + v2.im * v2.im + v3.re * v3.re + v3.im * v3.im;
         nn = fmaf(q, m, nn);
         nd = fmaf(d.re, d.re, fmaf(d.im, d.im, nd));
       }
     }
-    if (MODE == CGF_STEP) {
+    if (MODE != CGF_INIT) {
       // Parseval over the half spectrum: columns 0 < kx < n1/2 stand for their conjugates too
       const float wt = !valid ? 0.0f : (kx == 0 || kx == g.h) ? 1.0f : 2.0f;
       sum_n += (double)(wt * nn);
@@ -426,7 +430,7 @@ __global__ void __launch_bounds__(ZLaunch<N, TC>::threads, ZLaunch<N, TC>::min_b
     atomicAdd(a.prof, (unsigned long long)((6 + (MODE == CGF_STEP ? 6 : 3)) * N * cols * (long long)sizeof(cx<float>)));
     atomicAdd(a.prof + 1, (unsigned long long)(N * cols));
   }
-  if (MODE == CGF_STEP) {
+  if (MODE != CGF_INIT) {
     // |e|^2 = 2 |q|^2 |v|^2 + 2 |q . v|^2 and tr e = 2 q . v give ||e||^2 and <e, e>_C0
     double* red = reinterpret_cast<double*>(smem_raw);
     __syncthreads();   // the exchange buffers are free
@@ -440,7 +444,7 @@ __global__ void __launch_bounds__(ZLaunch<N, TC>::threads, ZLaunch<N, TC>::min_b
       double vv[2] = {2.0 * mu0 * e2 + 4.0 * lam0 * sd, e2};
       const int ncta = gridDim.x;
       if (warp_publish_and_collect<2>(vv, a.part + (long long)rhs * 2 * ncta, a.cnt + rhs, ncta, blockIdx.x) && tid == 0)
-        finalize_state(FIN_CG, a.st[rhs], vv, 1.0);
+        finalize_state(MODE == CGF_RHS ? FIN_RHS : FIN_CG, a.st[rhs], vv, 1.0);
     }
   }
 }
@@ -487,7 +491,9 @@ cudaError_t run_inv(const CgZArgs& a, int mode, int nrhs, cudaStream_t s) {
 }
 template <int N, int TC>
 cudaError_t run_fwd(const CgZArgs& a, int mode, int nrhs, cudaStream_t s) {
-  return mode == CGF_STEP ? run_fwd_mode<N, TC, CGF_STEP>(a, nrhs, s) : run_fwd_mode<N, TC, CGF_INIT>(a, nrhs, s);
+  return mode == CGF_STEP   ? run_fwd_mode<N, TC, CGF_STEP>(a, nrhs, s)
+         : mode == CGF_INIT ? run_fwd_mode<N, TC, CGF_INIT>(a, nrhs, s)
+                            : run_fwd_mode<N, TC, CGF_RHS>(a, nrhs, s);
 }
 
 #ifndef HOM_Z_LENGTHS
@@ -501,6 +507,7 @@ long long cg_vector_elems(const Geo& g) {
   const int tc = tile_width(g);
   return (g.plane_c + tc - 1) / tc * tc * 3 * g.n3;
 }
+int cg_vector_tile(const Geo& g) { return tile_width(g); }
 int cg_z_blocks(const Geo& g) {
   const int tc = tile_width(g);
   const long long tiles = (g.plane_c + tc - 1) / tc, group = tile_group(g, tc);

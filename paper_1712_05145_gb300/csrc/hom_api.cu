@@ -209,8 +209,12 @@ hom_status work(hom_ctx* c, int i, size_t bytes, void** out) {
 // partial sums one load's reducing kernel publishes at most (one per CTA)
 size_t ncta_max(const hom_ctx* c) {
   size_t m = 6 * (size_t)std::max(c->g.n3 * std::max(1, c->g.pc_Q), c->g.split ? c->g.nrb : 0);
-  if (c->fp32)   // the CG passes in Fourier space: row blocks and z tiles
+  if (c->fp32) {   // the CG passes in Fourier space: row blocks and z tiles, and the double-float z tiles
     m = std::max(m, std::max(6 * (size_t)cg_row_blocks(c->g), (size_t)cg_z_blocks(c->g)));
+    ZArgs<df64> t{};
+    t.g = c->g;
+    if (zcluster_tiling<df64>(t, -1)) m = std::max(m, 6 * (size_t)t.ntiles);
+  }
   return m + 64;
 }
 
@@ -697,27 +701,85 @@ hom_status cg_iterations(hom_ctx* c, CgPass& q, int r0, int m, int iters) {
   return HOM_OK;
 }
 
+// Launch arguments of the double-float z passes around FP32 CG sweeps; false on grids too shallow for
+// their tiles (N3 < 16), which take the real-space passes instead
+bool cg_df_args(hom_ctx* c, cx<float>* rh, const cx<float>* ph, const cx<float>* xh, CgDfArgs& a) {
+  ZArgs<df64> t{};
+  t.g = c->g;
+  if (!zcluster_tiling<df64>(t, -1)) return false;
+  a = CgDfArgs{};
+  a.g = c->g;
+  a.r = rh;
+  a.p = ph;
+  a.x = xh;
+  const int tc = cg_vector_tile(c->g);
+  while ((1 << a.vec_lg) < tc) ++a.vec_lg;
+  a.vec_tiles = (int)((c->g.plane_c + tc - 1) / tc);
+  a.st = c->d_st;
+  a.lam0 = c->lam0;
+  a.mu0 = c->mu0;
+  a.rve_loads = c->rve_loads;
+  a.c0 = c->rve_loads > 0 ? c->d_c0 : nullptr;
+  a.scale = 1.0 / (double)c->g.M;
+  a.green = c->opt.green_operator;
+  a.gtab = c->d_gtab;
+  a.tw_n3 = tw<df64>(c, 3);
+  a.tc_log2 = t.tc_log2;
+  a.ntiles = t.ntiles;
+  a.nthr = t.nthr;
+  a.fd_in = t.fd_in;
+  a.part = part_inv(c);
+  a.cnt = cnt_inv(c);
+  a.prof = c->prof_on ? c->d_prof + 2 * HOM_KERNEL_ZPASS_F64 : nullptr;
+  return true;
+}
+
+bool any_of(const std::vector<int>& v, int r0, int m) {
+  for (int i = r0; i < r0 + m; ++i)
+    if (v[i]) return true;
+  return false;
+}
+
+// rh = b - Gamma0 * (C : (x64 + E)) in Fourier space, with its norms (fin: FIN_RESID or FIN_RHS), at FP64
+// accuracy (see cg_df.cu); x64 = nullptr: x = 0, b64 = nullptr: b is the E term
+hom_status cg_residual_fourier(hom_ctx* c, int n, const double* dE, const double* b64, const double* x64, CgDfArgs da,
+                               int fin, const std::vector<int>& act) {
+  int chunk;
+  cx<df64>* S = spec<df64>(c, &chunk);
+  auto fa = fwd_args<double, df64>(c, FWD_STRESS, 6, 6);
+  fa.in = x64;
+  fa.E = dE;
+  fa.bsub = b64;
+  fa.st = c->d_st;
+  fa.S = da.S = S;
+  da.fin = fin;
+  for (int r0 = 0; r0 < n; r0 += chunk) {
+    const int m = std::min(chunk, n - r0);
+    if (!any_of(act, r0, m)) continue;
+    fa.rhs0 = da.rhs0 = r0;
+    CKS((fwd_xy<double, df64>(c, fa, m)));
+    CKS(timed_launch(c, HOM_KERNEL_ZPASS_F64, [&] { return launch_cg_df_residual(da, m, c->stream); }));
+  }
+  return HOM_OK;
+}
+
 // One FP32 CG sweep on A d = r (Eq. cg_form) with its vectors in Fourier space, for the active loads:
-// r (real, compatible) goes to rh, CG runs until every load's device state is inactive, and the
-// correction d is added to x64.  rh, ph, xh: n loads' vectors (hat_bytes); ph may be r's buffer, which
-// is read before the first iteration writes p.  A chunk of loads runs check_every iterations before the
-// next chunk starts, so that vectors that fit the L2 cache stay there.
+// r (real, compatible; nullptr if rh holds it already) goes to rh, CG runs until every load's device
+// state is inactive, and the correction d is added to x64, through double-float transforms if df is
+// given.  rh, ph, xh: n loads' vectors (hat_bytes); ph may be r's buffer, which is read before the first
+// iteration writes p.  A chunk of loads runs check_every iterations before the next chunk starts, so
+// that vectors that fit the L2 cache stay there.
 hom_status cg_sweep_fourier(hom_ctx* c, int n, const float* r, cx<float>* rh, cx<float>* ph, cx<float>* xh,
-                            double* x64, std::vector<RhsState>& st, std::vector<int>& act) {
+                            double* x64, CgDfArgs* df, std::vector<RhsState>& st, std::vector<int>& act) {
   const std::vector<int> ran = act;
   const int chunk = c->chunk;
   CgPass q = cg_pass(c, rh, ph, xh);
-  auto any_of = [&](const std::vector<int>& v, int r0, int m) {
-    for (int i = r0; i < r0 + m; ++i)
-      if (v[i]) return true;
-    return false;
-  };
   // r -> rh
   auto fa = fwd_args<float, float>(c, FWD_COPY, 6, 6);
   fa.in = r;
   fa.st = c->d_st;
   fa.S = q.za.S;
-  for (int r0 = 0; r0 < n; r0 += chunk) {
+  for (int r0 = 0; r != nullptr && r0 < n; r0 += chunk) {
     const int m = std::min(chunk, n - r0);
     if (!any_of(act, r0, m)) continue;
     fa.rhs0 = q.za.rhs0 = r0;
@@ -741,16 +803,32 @@ hom_status cg_sweep_fourier(hom_ctx* c, int n, const float* r, cx<float>* rh, cx
   // x64 += d, with the update of x that the last iteration left pending
   for (int i = 0; i < n; ++i) st[i].active = ran[i];
   CKS(write_states(c, st));
-  auto ia = inv_args<double, float>(c, INV_ADD, FIN_NONE, 6, 6, 6);
-  ia.S = q.za.S;
-  ia.st = c->d_st;
-  ia.out = x64;
-  for (int r0 = 0; r0 < n; r0 += chunk) {
-    const int m = std::min(chunk, n - r0);
-    if (!any_of(ran, r0, m)) continue;
-    q.za.rhs0 = ia.rhs0 = r0;
-    CKS(timed_launch(c, HOM_KERNEL_ZPASS, [&] { return launch_cg_z_inv(q.za, CGI_OUT, m, c->stream); }));
-    CKS((inv_xy<double, float>(c, ia, m)));
+  if (df != nullptr) {
+    int chunk64;
+    auto ia = inv_args<double, df64>(c, INV_STORE, FIN_NONE, 6, 6, 6);   // x64 = d + x64
+    ia.S = df->S = spec<df64>(c, &chunk64);
+    ia.st = c->d_st;
+    ia.b = x64;
+    ia.out = x64;
+    for (int r0 = 0; r0 < n; r0 += chunk64) {
+      const int m = std::min(chunk64, n - r0);
+      if (!any_of(ran, r0, m)) continue;
+      df->rhs0 = ia.rhs0 = r0;
+      CKS(timed_launch(c, HOM_KERNEL_ZPASS_F64, [&] { return launch_cg_df_out(*df, m, c->stream); }));
+      CKS((inv_xy<double, df64>(c, ia, m)));
+    }
+  } else {
+    auto ia = inv_args<double, float>(c, INV_ADD, FIN_NONE, 6, 6, 6);
+    ia.S = q.za.S;
+    ia.st = c->d_st;
+    ia.out = x64;
+    for (int r0 = 0; r0 < n; r0 += chunk) {
+      const int m = std::min(chunk, n - r0);
+      if (!any_of(ran, r0, m)) continue;
+      q.za.rhs0 = ia.rhs0 = r0;
+      CKS(timed_launch(c, HOM_KERNEL_ZPASS, [&] { return launch_cg_z_inv(q.za, CGI_OUT, m, c->stream); }));
+      CKS((inv_xy<double, float>(c, ia, m)));
+    }
   }
   for (int i = 0; i < n; ++i) {
     st[i].xpend = 0;
@@ -1186,7 +1264,7 @@ hom_status solve_system(hom_ctx* c, int n, const double* dE, const double* b64, 
   // The first sweep starts from b and aims at the tolerance itself where FP32 can reach it
   // (relative residuals down to kFirstSweepFloor); later sweeps ask for kSweepGain relative to
   // the FP64 residual they restart from.
-  const double kSweepGain = 1e-5, kFirstSweepTarget = 1e-4;
+  const double kSweepGain = 1e-5, kFirstSweepTarget = 1e-4, kFp32OutTol = 5e-7;
   const double tol_inner = (mixed && !basic) ? std::max(0.5 * tol, kFirstSweepTarget) : (mixed ? 0.5 * tol : tol);
   // FP32 corrections computed on real fields (BiCGSTAB) leave an incompatible part in x: step lengths
   // reach C0 / C_min along the soft phases' directions and multiply the FP32 rounding of each direction
@@ -1285,8 +1363,28 @@ hom_status solve_system(hom_ctx* c, int n, const double* dE, const double* b64, 
   } else {
     CK(cudaMemsetAsync(x64, 0, tbytes<double>(c, n, 6), c->stream));
     if (mixed && !fourier) CK(cudaMemsetAsync(d, 0, fb, c->stream));
-    // initial residual r = b (x = 0)
-    if (dE != nullptr) {
+    // initial residual r = b (x = 0); FP32 CG takes it (and every restart's) in Fourier space
+    bool have_rh = false;   // the CG vector r holds the residual, not the real field
+    CgDfArgs df;
+    const bool df_z = fourier && cg_df_args(c, reinterpret_cast<cx<float>*>(vp), reinterpret_cast<cx<float>*>(vr),
+                                            reinterpret_cast<cx<float>*>(vd), df);
+    if (fourier && dE != nullptr) {
+      CgPass q = cg_pass(c, reinterpret_cast<cx<float>*>(vp), nullptr, nullptr);
+      auto fa = fwd_args<float, float>(c, FWD_TAU, 6, 6);
+      fa.E = dE;
+      fa.st = c->d_st;
+      fa.S = q.za.S;
+      for (int r0 = 0; r0 < n; r0 += c->chunk) {
+        const int m = std::min(c->chunk, n - r0);
+        fa.rhs0 = q.za.rhs0 = r0;
+        CKS((fwd_xy<float, float>(c, fa, m)));
+        CKS(timed_launch(c, HOM_KERNEL_ZPASS, [&] { return launch_cg_z_fwd(q.za, CGF_RHS, m, c->stream); }));
+      }
+      have_rh = true;
+    } else if (df_z) {
+      CKS(cg_residual_fourier(c, n, nullptr, b64, nullptr, df, FIN_RHS, act));
+      have_rh = true;
+    } else if (dE != nullptr) {
       auto fa = fwd_args<Tf, Tf>(c, FWD_TAU, 6, 6);
       fa.E = dE;
       fa.st = c->d_st;
@@ -1310,7 +1408,7 @@ hom_status solve_system(hom_ctx* c, int n, const double* dE, const double* b64, 
       }
     }
     CKS(write_states(c, st));
-    while (true) {
+    for (int sweep = 0;; ++sweep) {
       bool any = false;
       for (int i = 0; i < n; ++i) any = any || act[i];
       if (bicg && any) {
@@ -1323,8 +1421,12 @@ hom_status solve_system(hom_ctx* c, int n, const double* dE, const double* b64, 
       }
       if constexpr (std::is_same<Tf, float>::value) {
         if (any) {
-          CKS(cg_sweep_fourier(c, n, r, reinterpret_cast<cx<float>*>(vp), reinterpret_cast<cx<float>*>(vr),
-                               reinterpret_cast<cx<float>*>(vd), x64, st, act));
+          // a tight tolerance sees the incompatible rounding that an FP32 transform of the whole solution
+          // leaves (about 1e-7 of ||x||): the first sweep's correction is then added in double-float
+          const bool exact_out = df_z && sweep == 0 && tol < kFp32OutTol;
+          CKS(cg_sweep_fourier(c, n, have_rh ? nullptr : r, reinterpret_cast<cx<float>*>(vp),
+                               reinterpret_cast<cx<float>*>(vr), reinterpret_cast<cx<float>*>(vd), x64,
+                               exact_out ? &df : nullptr, st, act));
           any = false;
         }
       }
@@ -1422,7 +1524,9 @@ hom_status solve_system(hom_ctx* c, int n, const double* dE, const double* b64, 
         for (int i = 0; i < n; ++i) st[i].active = act[i];
         CKS(write_states(c, st));
       }
-      CKS(residual_sweep<Tf>(c, n, dE, b64, x64, r, FIN_RESID, &act));
+      if (df_z) CKS(cg_residual_fourier(c, n, dE, b64, x64, df, FIN_RESID, act));
+      else CKS(residual_sweep<Tf>(c, n, dE, b64, x64, r, FIN_RESID, &act));
+      have_rh = df_z;
       CKS(read_states(c, n, st));
       bool again = false;
       for (int i = 0; i < n; ++i) {

@@ -88,6 +88,7 @@ struct FwdArgs {
   const double* c0;            // rve_loads > 0: [rve][4] (lambda0, mu0, 3 lambda0 + 2 mu0, 2 mu0) per RVE
   const Tf* in;                // FWD_TAU: strain (nullable); FWD_COPY: field
   const double* E;             // FWD_TAU: [rhs][6] Kelvin macroscopic strain (nullable)
+  const double* bsub;          // FWD_STRESS in double-float: tau -= C0 : bsub (nullable), [rhs][6][M]
   const Tf* r;                 // FWD_CG
   Tf* p;                       // FWD_CG (read old p, write new p)
   Tf* x;                       // FWD_CG (x += alpha p with the old p, except at a restart)

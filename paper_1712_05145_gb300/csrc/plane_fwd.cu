@@ -75,6 +75,9 @@ plane_fwd_kernel(const FwdArgs<Tf, T> a) {
   if (a.mode == FWD_TAU || a.mode == FWD_STRESS) {
     const T ec = (a.E != nullptr) ? (T)a.E[rhs * 6 + c] : (T)0;
     const T* w = (a.mode == FWD_TAU) ? tab : tab + a.n_phase;
+    T ch, cd;
+    c0_weights<T>(a.c0, rve, a.c0h, a.c0d, ch, cd);
+    const T wb = (c == 0) ? ch : cd;   // C0 on this component, for bsub
     #pragma unroll 4
     for (int row = warp; row < n2; row += nwarp) {
       for (int c2 = lane; c2 < h; c2 += 32) {
@@ -82,7 +85,16 @@ plane_fwd_kernel(const FwdArgs<Tf, T> a) {
         Tf v0 = 0, v1 = 0;
         if (a.in != nullptr) ld2<Tf>(a.in + foff + o, v0, v1);
         const uchar2 ph = *reinterpret_cast<const uchar2*>(php + o);
-        pl[row * P + c2] = mk<T>(w[ph.x] * ((T)v0 + ec), w[ph.y] * ((T)v1 + ec));
+        T t0 = w[ph.x] * ((T)v0 + ec), t1 = w[ph.y] * ((T)v1 + ec);
+        if constexpr (std::is_same<T, df64>::value) {
+          if (a.bsub != nullptr) {
+            double b0, b1;
+            ld2<double>(a.bsub + foff + o, b0, b1);
+            t0 -= wb * (T)b0;
+            t1 -= wb * (T)b1;
+          }
+        }
+        pl[row * P + c2] = mk<T>(t0, t1);
       }
     }
   } else if (kRealCg<T> && a.mode == FWD_CG) {

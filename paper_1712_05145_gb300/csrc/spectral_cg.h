@@ -35,9 +35,40 @@ struct CgZArgs {
   unsigned long long* prof;
 };
 // cg_z_inv: CGI_STEP the iteration's first pass; CGI_OUT x += alpha p where pending, strain of x -> S
-// cg_z_fwd: CGF_STEP the iteration's last pass; CGF_INIT r = the components v of a compatible strain
+// cg_z_fwd: CGF_STEP the iteration's last pass; CGF_INIT r = the components v of a compatible strain;
+//           CGF_RHS r = -Gamma0_hat : tau_hat with its norms (the right-hand side, from tau = (C - C0) : E)
 enum CgInvMode { CGI_STEP = 0, CGI_OUT = 1 };
-enum CgFwdMode { CGF_STEP = 0, CGF_INIT = 1 };
+enum CgFwdMode { CGF_STEP = 0, CGF_INIT = 1, CGF_RHS = 2 };
+
+// z passes in double-float around a sweep (cg_df.cu), with the tiles of the cluster z pass
+struct CgDfArgs {
+  Geo g;
+  cx<df64>* S;             // chunk spectrum [load][6][n3][plane_c]
+  cx<float>* r;            // cg_df_residual writes r
+  const cx<float>* p;      // cg_df_out reads x and p
+  const cx<float>* x;
+  int vec_lg;              // log2 of the vectors' tile width, and tiles per load (cg_vector_tile)
+  int vec_tiles;
+  int rhs0;
+  RhsState* st;
+  int fin;                 // cg_df_residual: FIN_RHS or FIN_RESID
+  double lam0, mu0;
+  int rve_loads;
+  const double* c0;
+  double scale;            // 1 / M
+  int green;
+  const double* gtab;
+  const cx<df64>* tw_n3;
+  int tc_log2, ntiles, nthr;   // tiling of zcluster_tiling<df64>
+  FastDiv fd_in;
+  double* part;            // cg_df_residual: [rhs][2][6 ntiles]
+  unsigned* cnt;
+  unsigned long long* prof;
+};
+// r = -v(tau_hat) and its norms, from the x-y transforms of tau = C : (x + E) - C0 : b: r = b - Gamma0 * (C : (x + E))
+cudaError_t launch_cg_df_residual(const CgDfArgs& a, int nrhs, cudaStream_t s);
+// strain of x (with its pending update), inverse z FFT -> S
+cudaError_t launch_cg_df_out(const CgDfArgs& a, int nrhs, cudaStream_t s);
 
 struct CgPlaneArgs {
   Geo g;
@@ -57,6 +88,7 @@ struct CgPlaneArgs {
 };
 
 long long cg_vector_elems(const Geo& g);  // complex values of one load's vector
+int cg_vector_tile(const Geo& g);         // columns of one of its tiles (a power of two)
 int cg_z_blocks(const Geo& g);            // CTAs of one load in the z passes
 cudaError_t launch_cg_z_inv(const CgZArgs& a, int mode, int nrhs, cudaStream_t s);
 cudaError_t launch_cg_z_fwd(const CgZArgs& a, int mode, int nrhs, cudaStream_t s);

@@ -148,6 +148,15 @@ __global__ void __launch_bounds__(256 * (kEPT / EPT), XfCfg<T>::kMinBlocks) xpas
             if (a.in != nullptr) ld2<Tf>(a.in + cbase + o, v0, v1);
             const uchar2 ph = *reinterpret_cast<const uchar2*>(phase + o);
             val = mk<T>(w[ph.x] * ((T)v0 + ec), w[ph.y] * ((T)v1 + ec));
+            if constexpr (std::is_same<T, df64>::value) {
+              if (a.bsub != nullptr) {
+                const T wb = (c == 0) ? ch : cd;
+                double b0, b1;
+                ld2<double>(a.bsub + cbase + o, b0, b1);
+                val.re -= wb * (T)b0;
+                val.im -= wb * (T)b1;
+              }
+            }
           } else {
             Tf v0, v1;
             ld2<Tf>(a.in + cbase + o, v0, v1);
