@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(512, 2) cg_plane_kernel(const CgPlaneArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const Geo& g = a.g;
   const int z = blockIdx.x, c = blockIdx.y, lrhs = blockIdx.z, rhs = a.rhs0 + lrhs;
-  if (a.st[rhs].active == 0) return;
+  grid_dep_launch();
   constexpr int h = H, n1 = 2 * H, P = kPitch<H>;
   const int n2 = g.n2;
   PlaneSmem m;
@@ -259,6 +259,8 @@ __global__ void __launch_bounds__(512, 2) cg_plane_kernel(const CgPlaneArgs a) {
     }
   }
   __syncthreads();
+  grid_dep_wait();
+  if (a.st[rhs].active == 0) return;
   cx<float>* Sp = a.S + ((long long)(lrhs * 6 + c) * g.n3 + z) * g.plane_c;
   // planes of at most kMaxPlane values: larger pairs of lengths are not instantiated
   switch (n2) {
@@ -306,8 +308,7 @@ cudaError_t run_plane(const CgPlaneArgs& a, int nrhs, cudaStream_t s) {
                       (256 + thr) * sizeof(float) + (size_t)g.n2 * (g.n1 + 4);
   cudaError_t err = set_smem(cg_plane_kernel<H>, smem);
   if (err != cudaSuccess) return err;
-  cg_plane_kernel<H><<<dim3(g.n3, 6, nrhs), thr, smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_dependent(cg_plane_kernel<H>, dim3(g.n3, 6, nrhs), thr, smem, s, a);
 }
 
 }  // namespace

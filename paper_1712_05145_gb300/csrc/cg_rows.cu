@@ -29,7 +29,7 @@ __global__ void __launch_bounds__(kRowThreads, 4) cg_rows_kernel(const CgPlaneAr
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const Geo& g = a.g;
   const int c = blockIdx.y, lrhs = blockIdx.z, rhs = a.rhs0 + lrhs;
-  if (a.st[rhs].active == 0) return;
+  grid_dep_launch();
   cx<float>* pl = reinterpret_cast<cx<float>*>(smem_raw);
   cx<float>* twh = pl + ROWS * RB::pitch;
   cx<float>* tw1 = twh + H;
@@ -47,6 +47,8 @@ __global__ void __launch_bounds__(kRowThreads, 4) cg_rows_kernel(const CgPlaneAr
   const float* mat = a.mat + (long long)rve * kRveTable;
   for (int i = tid; i < a.n_phase; i += kRowThreads) tab[i] = 0.5f * mat[i * 4 + (c == 0 ? 2 : 3)];
   __syncthreads();
+  grid_dep_wait();
+  if (a.st[rhs].active == 0) return;
   // row r of the block: start of its half spectrum in S
   auto row_ptr = [&](int r) {
     const unsigned gr = row0 + (unsigned)r, z = g.fd_n2.div(gr), y = gr - z * (unsigned)g.n2;
@@ -132,8 +134,7 @@ template <int H>
 cudaError_t run_rows(const CgPlaneArgs& a, int nrhs, cudaStream_t s) {
   cudaError_t e = set_smem(cg_rows_kernel<H>, RowBlock<H>::smem);
   if (e != cudaSuccess) return e;
-  cg_rows_kernel<H><<<dim3(cg_row_blocks(a.g), 6, nrhs), kRowThreads, RowBlock<H>::smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_dependent(cg_rows_kernel<H>, dim3(cg_row_blocks(a.g), 6, nrhs), kRowThreads, RowBlock<H>::smem, s, a);
 }
 
 #define HOM_ROW_LENGTHS(X) \

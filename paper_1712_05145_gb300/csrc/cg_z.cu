@@ -137,24 +137,28 @@ template <int N, int TC> struct ZLaunch {
 struct ColumnQ {
   float a1, a2, a3;
 };
-__device__ __forceinline__ ColumnQ column_q(const Geo& g, int green, const double* gtab, int kx, int ky) {
+// (In FP32 throughout: a warp instruction takes 16 cycles of the SM's FP64 pipe, and these run in every thread.)
+__device__ __forceinline__ ColumnQ column_q(const CgZArgs& a, int kx, int ky) {
+  const Geo& g = a.g;
   ColumnQ q;
-  if (green == 0) {
-    q.a1 = (float)((kx == g.h ? 0 : kx) * g.xs1);
-    q.a2 = (float)(wave(ky, g.n2) * g.xs2);
+  if (a.green == 0) {
+    q.a1 = (float)(kx == g.h ? 0 : kx) * a.xs[0];
+    q.a2 = (float)wave(ky, g.n2) * a.xs[1];
     q.a3 = 1.0f;
   } else {
-    const double* t2 = gtab + 2 * (g.h + 1);
-    const double s1 = __ldg(gtab + kx), c1 = __ldg(gtab + g.h + 1 + kx), s2 = __ldg(t2 + ky), c2 = __ldg(t2 + g.n2 + ky);
-    q.a1 = (float)(s1 * c2);
-    q.a2 = (float)(c1 * s2);
-    q.a3 = (float)(c1 * c2);
+    const double* t2 = a.gtab + 2 * (g.h + 1);
+    const float s1 = (float)__ldg(a.gtab + kx), c1 = (float)__ldg(a.gtab + g.h + 1 + kx);
+    const float s2 = (float)__ldg(t2 + ky), c2 = (float)__ldg(t2 + g.n2 + ky);
+    q.a1 = s1 * c2;
+    q.a2 = c1 * s2;
+    q.a3 = c1 * c2;
   }
   return q;
 }
-__device__ __forceinline__ cx<float> z_factors(const Geo& g, int green, const double* gtab, int n) {   // (cz, sz)
-  if (green == 0) return mk<float>(1.0f, (float)(wave(n, g.n3) * g.xs3));
-  const double* t3 = gtab + 2 * (g.h + 1) + 2 * g.n2;
+__device__ __forceinline__ cx<float> z_factors(const CgZArgs& a, int n) {   // (cz, sz)
+  const Geo& g = a.g;
+  if (a.green == 0) return mk<float>(1.0f, (float)wave(n, g.n3) * a.xs[2]);
+  const double* t3 = a.gtab + 2 * (g.h + 1) + 2 * g.n2;
   return mk<float>((float)__ldg(t3 + g.n3 + n), (float)__ldg(t3 + n));
 }
 
@@ -224,8 +228,7 @@ __global__ void __launch_bounds__(ZLaunch<N, TC>::threads, ZLaunch<N, TC>::min_b
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const Geo& g = a.g;
   const int lrhs = blockIdx.y, rhs = a.rhs0 + lrhs;
-  const RhsState& s = a.st[rhs];
-  if (s.active == 0) return;
+  grid_dep_launch();
   cx<float>* b0 = reinterpret_cast<cx<float>*>(smem_raw);
   cx<float>* b1 = b0 + ZSmem<N, TC>::kBuf;
   cx<float>* tw = b0 + ZSmem<N, TC>::kArea;
@@ -233,8 +236,11 @@ __global__ void __launch_bounds__(ZLaunch<N, TC>::threads, ZLaunch<N, TC>::min_b
   const int tid = threadIdx.x, tc = tid % TC, u = tid / TC;
   for (int i = tid; i < N; i += THREADS) {
     tw[i] = ldg_cx(a.tw_n3 + i);
-    zt[i] = z_factors(g, a.green, a.gtab, i);
+    zt[i] = z_factors(a, i);
   }
+  grid_dep_wait();
+  const RhsState& s = a.st[rhs];
+  if (s.active == 0) return;
   const unsigned pc = (unsigned)g.plane_c;
   const size_t comp = (size_t)N * pc;
   const bool restart = s.restart != 0;
@@ -249,7 +255,7 @@ __global__ void __launch_bounds__(ZLaunch<N, TC>::threads, ZLaunch<N, TC>::min_b
     const bool valid = f < pc;
     int kx, ky;
     column_of(g, f, valid, kx, ky);
-    const ColumnQ cq = column_q(g, a.green, a.gtab, kx, ky);
+    const ColumnQ cq = column_q(a, kx, ky);
     // element e = b * RF + r of this thread is plane u + b U + r N / RF
     cx<float> v[3][E];
     const size_t block = ((size_t)rhs * ntiles + tile) * (3 * N * TC);
@@ -320,7 +326,7 @@ __global__ void __launch_bounds__(ZLaunch<N, TC>::threads, ZLaunch<N, TC>::min_b
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const Geo& g = a.g;
   const int lrhs = blockIdx.y, rhs = a.rhs0 + lrhs;
-  if (a.st[rhs].active == 0) return;
+  grid_dep_launch();
   cx<float>* b0 = reinterpret_cast<cx<float>*>(smem_raw);
   cx<float>* b1 = b0 + ZSmem<N, TC>::kBuf;
   cx<float>* tw = b0 + ZSmem<N, TC>::kArea;
@@ -342,27 +348,34 @@ __global__ void __launch_bounds__(ZLaunch<N, TC>::threads, ZLaunch<N, TC>::min_b
       for (int e = 0; e < E; ++e) nx[e] = mk<float>(0.0f, 0.0f);
     }
   };
-  fetch(blockIdx.x, 0);
   for (int i = tid; i < N; i += THREADS) {
     tw[i] = ldg_cx(a.tw_n3 + i);
-    zt[i] = z_factors(g, a.green, a.gtab, i);
+    zt[i] = z_factors(a, i);
   }
   // v = Gamma0_hat(q) : tau_hat from w = tau_hat q (STEP, RHS), or the components of a compatible strain (INIT)
-  float c1 = 1.0f, c2h = 0.5f;
+  __shared__ float gc[2];
   const int rve = rve_of(rhs, a.rve_loads);
-  if (MODE != CGF_INIT) green_consts<float>(a.c0, rve, a.lam0, a.mu0, c1, c2h);
-  c1 *= a.scale;
-  c2h *= a.scale;
+  if (tid == 0) {   // two FP64 divisions: one thread's
+    float c1 = 1.0f, c2h = 0.5f;
+    if (MODE != CGF_INIT) green_consts<float>(a.c0, rve, a.lam0, a.mu0, c1, c2h);
+    gc[0] = c1 * a.scale;
+    gc[1] = c2h * a.scale;
+  }
+  grid_dep_wait();
+  const int active = a.st[rhs].active;
+  fetch(blockIdx.x, 0);   // with the state on its way: a launch rarely holds loads that have ended
+  if (active == 0) return;
   const float alpha = MODE == CGF_STEP ? (float)a.st[rhs].alpha : 0.0f;
   double sum_n = 0.0, sum_d = 0.0;   // weighted sums of |q|^2 |v|^2 and |q . v|^2 over the new r
   __syncthreads();   // tables
+  const float c1 = gc[0], c2h = gc[1];
 #pragma unroll 1
   for (int tile = blockIdx.x; tile < ntiles; tile += step) {
     const unsigned f = (unsigned)tile * TC + tc;
     const bool valid = f < pc;
     int kx, ky;
     column_of(g, f, valid, kx, ky);
-    const ColumnQ cq = column_q(g, a.green, a.gtab, kx, ky);
+    const ColumnQ cq = column_q(a, kx, ky);
     cx<float>* rl = a.r + ((size_t)rhs * ntiles + tile) * (3 * N * TC);
     // this tile's r, needed after the transforms
     if (MODE == CGF_STEP && tid == 0) prefetch_l2(rl, 3 * N * TC * sizeof(cx<float>));
@@ -472,18 +485,16 @@ cudaError_t run_inv_mode(const CgZArgs& a, int nrhs, cudaStream_t s) {
   const int tiles = (int)((a.g.plane_c + TC - 1) / TC), group = tile_group(a.g, TC);
   cudaError_t e = set_smem(cg_z_inv_kernel<N, TC, MODE>, ZSmem<N, TC>::bytes);
   if (e != cudaSuccess) return e;
-  cg_z_inv_kernel<N, TC, MODE><<<dim3((unsigned)((tiles + group - 1) / group), (unsigned)nrhs), ZLaunch<N, TC>::threads,
-                                 ZSmem<N, TC>::bytes, s>>>(a, tiles);
-  return cudaGetLastError();
+  return launch_dependent(cg_z_inv_kernel<N, TC, MODE>, dim3((unsigned)((tiles + group - 1) / group), (unsigned)nrhs),
+                          ZLaunch<N, TC>::threads, ZSmem<N, TC>::bytes, s, a, tiles);
 }
 template <int N, int TC, int MODE>
 cudaError_t run_fwd_mode(const CgZArgs& a, int nrhs, cudaStream_t s) {
   const int tiles = (int)((a.g.plane_c + TC - 1) / TC), group = tile_group(a.g, TC);
   cudaError_t e = set_smem(cg_z_fwd_kernel<N, TC, MODE>, ZSmem<N, TC>::bytes);
   if (e != cudaSuccess) return e;
-  cg_z_fwd_kernel<N, TC, MODE><<<dim3((unsigned)((tiles + group - 1) / group), (unsigned)nrhs), ZLaunch<N, TC>::threads,
-                                 ZSmem<N, TC>::bytes, s>>>(a, tiles);
-  return cudaGetLastError();
+  return launch_dependent(cg_z_fwd_kernel<N, TC, MODE>, dim3((unsigned)((tiles + group - 1) / group), (unsigned)nrhs),
+                          ZLaunch<N, TC>::threads, ZSmem<N, TC>::bytes, s, a, tiles);
 }
 template <int N, int TC>
 cudaError_t run_inv(const CgZArgs& a, int mode, int nrhs, cudaStream_t s) {

@@ -655,6 +655,9 @@ CgPass cg_pass(hom_ctx* c, cx<float>* rh, cx<float>* ph, cx<float>* xh) {
   za.rve_loads = c->rve_loads;
   za.c0 = c->rve_loads > 0 ? c->d_c0 : nullptr;
   za.scale = (float)(1.0 / (double)c->g.M);
+  za.xs[0] = (float)c->g.xs1;
+  za.xs[1] = (float)c->g.xs2;
+  za.xs[2] = (float)c->g.xs3;
   za.green = c->opt.green_operator;
   za.gtab = c->d_gtab;
   za.tw_n3 = tw<float>(c, 3);

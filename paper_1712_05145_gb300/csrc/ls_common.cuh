@@ -279,13 +279,34 @@ inline int smem_optin_max() {
   return v;
 }
 
+// Programmatic dependent launch.  A kernel launched with launch_dependent starts while its predecessor in
+// the stream still runs, once all of the predecessor's CTAs have called grid_dep_launch or ended; what it
+// does before grid_dep_wait overlaps the predecessor's tail and may read constants only.  Every CTA waits
+// before it ends, also one that has nothing to do: the kernel after the next one relies on it.
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <typename... P, typename... A>
+inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 template <typename K>
 inline cudaError_t set_smem(K kernel, size_t bytes) {
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                        (int)cudaSharedmemCarveoutMaxShared);
   if (e != cudaSuccess) return e;
   if (bytes <= 48 * 1024) return cudaSuccess;
-  const int optin = smem_optin_max();
+  const int optin = smem_optin_max() - 1024;   // the limit includes a kernel's static shared memory (below 1 KB here)
   if ((long long)bytes > optin) return cudaErrorInvalidValue;
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
 }

@@ -27,6 +27,7 @@ struct CgZArgs {
   int rve_loads;
   const double* c0;        // several RVE slots: [rve][4], see ZArgs
   float scale;             // 1 / M, the factor of the forward transform
+  float xs[3];             // Geo's xs1, xs2, xs3
   int green;
   const double* gtab;
   const cx<float>* tw_n3;
