@@ -48,8 +48,7 @@ __global__ void __cluster_dims__(6, 1, 1) __launch_bounds__(kDfThreads, 1) cg_df
   const long long f0 = (long long)tile * TC;
   cx<df64>* buf = reinterpret_cast<cx<df64>*>(smem_raw);   // [n3][TC]
   cx<df64>* twz = buf + per;
-  double* sh = reinterpret_cast<double*>(twz + n3);
-  int* flag = reinterpret_cast<int*>(sh + 64);
+  double* red = reinterpret_cast<double*>(twz + n3);       // [2][threads]
   const int tid = threadIdx.x, nthr = blockDim.x;
   const cx<df64>* Sc = a.S + (long long)(lrhs * 6 + comp) * n3 * g.plane_c;
   for (int e = tid; e < per; e += nthr) {
@@ -63,6 +62,8 @@ __global__ void __cluster_dims__(6, 1, 1) __launch_bounds__(kDfThreads, 1) cg_df
     atomicAdd(a.prof, (unsigned long long)(n3 * cols * (long long)(sizeof(cx<df64>) + sizeof(cx<float>) / 2)));
     if (comp == 0) atomicAdd(a.prof + 1, (unsigned long long)(n3 * cols));
   }
+  __shared__ df64 gc[2];
+  green_consts_shared<df64>(gc, a.c0, rve_of(rhs, a.rve_loads), a.lam0, a.mu0);
   cp_async_wait_all();
   __syncthreads();
   fft_pencils<df64, -1, kDfEPT>(buf, ColAddr{TC}, n3, TC, a.fd_in, twz);
@@ -72,8 +73,7 @@ __global__ void __cluster_dims__(6, 1, 1) __launch_bounds__(kDfThreads, 1) cg_df
     const cx<df64>* part[6];
 #pragma unroll
     for (int r = 0; r < 6; ++r) part[r] = cl.map_shared_rank(buf, r);
-    df64 c1, c2h;
-    green_consts<df64>(a.c0, rve_of(rhs, a.rve_loads), a.lam0, a.mu0, c1, c2h);
+    const df64 c1 = gc[0], c2h = gc[1];
     const df64 scale = (df64)a.scale;
     const int share = (per + 5) / 6;
     const int q0 = comp * share, q1 = (q0 + share < per) ? q0 + share : per;
@@ -111,18 +111,17 @@ __global__ void __cluster_dims__(6, 1, 1) __launch_bounds__(kDfThreads, 1) cg_df
     }
   }
   // |e|^2 = 2 |q|^2 |v|^2 + 2 |q . v|^2 and tr e = 2 q . v, as in cg_z_fwd
-  double v[2] = {(double)nn, (double)nd};
-  block_sum_f64<2>(v, sh);
-  if (threadIdx.x == 0) {
-    const int rve = rve_of(rhs, a.rve_loads);
+  red[tid] = (double)nn;
+  red[nthr + tid] = (double)nd;
+  __syncthreads();
+  if (tid < 32) {
+    const double sn = warp_sum_f64(red, nthr), sd = warp_sum_f64(red + nthr, nthr);
+    const int rve = rve_of(rhs, a.rve_loads), ncta = gridDim.x;
     const double lam0 = a.c0 ? a.c0[4 * rve] : a.lam0, mu0 = a.c0 ? a.c0[4 * rve + 1] : a.mu0;
-    const double e2 = 2.0 * (v[0] + v[1]);
-    v[0] = 2.0 * mu0 * e2 + 4.0 * lam0 * v[1];
-    v[1] = e2;
-  }
-  const int ncta = gridDim.x;
-  if (publish_and_collect<2>(v, a.part + (long long)rhs * 2 * ncta, a.cnt + rhs, ncta, blockIdx.x, sh, flag)) {
-    if (threadIdx.x == 0) finalize_state(a.fin, a.st[rhs], v, 1.0);
+    const double e2 = 2.0 * (sn + sd);
+    double v[2] = {2.0 * mu0 * e2 + 4.0 * lam0 * sd, e2};
+    if (warp_publish_and_collect<2>(v, a.part + (long long)rhs * 2 * ncta, a.cnt + rhs, ncta, blockIdx.x) && tid == 0)
+      finalize_state(a.fin, a.st[rhs], v, 1.0);
   }
   cl.sync();   // the others have read this CTA's buffer
 }
@@ -183,8 +182,8 @@ __global__ void __launch_bounds__(kDfThreads, 1) cg_df_out_kernel(const CgDfArgs
   }
 }
 
-size_t df_smem(const Geo& g, int lg) {
-  return (((size_t)g.n3 << lg) + g.n3) * sizeof(cx<df64>) + 64 * sizeof(double) + 16;
+size_t df_smem(const CgDfArgs& a) {
+  return (((size_t)a.g.n3 << a.tc_log2) + a.g.n3) * sizeof(cx<df64>) + 2 * (size_t)a.nthr * sizeof(double);
 }
 bool df_args_ok(const CgDfArgs& a, int nrhs) {
   return nrhs >= 1 && a.nthr >= 32 && a.nthr <= kDfThreads && ((long long)a.g.n3 << a.tc_log2) <= (long long)kDfEPT * a.nthr &&
@@ -195,7 +194,7 @@ bool df_args_ok(const CgDfArgs& a, int nrhs) {
 
 cudaError_t launch_cg_df_residual(const CgDfArgs& a, int nrhs, cudaStream_t s) {
   if (!df_args_ok(a, nrhs)) return cudaErrorInvalidValue;
-  const size_t smem = df_smem(a.g, a.tc_log2);
+  const size_t smem = df_smem(a);
   cudaError_t e = set_smem(cg_df_residual_kernel, smem);
   if (e != cudaSuccess) return e;
   count_launch();
@@ -204,7 +203,7 @@ cudaError_t launch_cg_df_residual(const CgDfArgs& a, int nrhs, cudaStream_t s) {
 }
 cudaError_t launch_cg_df_out(const CgDfArgs& a, int nrhs, cudaStream_t s) {
   if (!df_args_ok(a, nrhs)) return cudaErrorInvalidValue;
-  const size_t smem = df_smem(a.g, a.tc_log2);
+  const size_t smem = df_smem(a);
   cudaError_t e = set_smem(cg_df_out_kernel, smem);
   if (e != cudaSuccess) return e;
   count_launch();

@@ -142,8 +142,8 @@ __device__ __forceinline__ ColumnQ column_q(const CgZArgs& a, int kx, int ky) {
   const Geo& g = a.g;
   ColumnQ q;
   if (a.green == 0) {
-    q.a1 = (float)(kx == g.h ? 0 : kx) * a.xs[0];
-    q.a2 = (float)wave(ky, g.n2) * a.xs[1];
+    q.a1 = wave_scaled<float>(g, 0, kx == g.h ? 0 : kx);
+    q.a2 = wave_scaled<float>(g, 1, wave(ky, g.n2));
     q.a3 = 1.0f;
   } else {
     const double* t2 = a.gtab + 2 * (g.h + 1);
@@ -157,7 +157,7 @@ __device__ __forceinline__ ColumnQ column_q(const CgZArgs& a, int kx, int ky) {
 }
 __device__ __forceinline__ cx<float> z_factors(const CgZArgs& a, int n) {   // (cz, sz)
   const Geo& g = a.g;
-  if (a.green == 0) return mk<float>(1.0f, (float)wave(n, g.n3) * a.xs[2]);
+  if (a.green == 0) return mk<float>(1.0f, wave_scaled<float>(g, 2, wave(n, g.n3)));
   const double* t3 = a.gtab + 2 * (g.h + 1) + 2 * g.n2;
   return mk<float>((float)__ldg(t3 + g.n3 + n), (float)__ldg(t3 + n));
 }
@@ -355,12 +355,8 @@ __global__ void __launch_bounds__(ZLaunch<N, TC>::threads, ZLaunch<N, TC>::min_b
   // v = Gamma0_hat(q) : tau_hat from w = tau_hat q (STEP, RHS), or the components of a compatible strain (INIT)
   __shared__ float gc[2];
   const int rve = rve_of(rhs, a.rve_loads);
-  if (tid == 0) {   // two FP64 divisions: one thread's
-    float c1 = 1.0f, c2h = 0.5f;
-    if (MODE != CGF_INIT) green_consts<float>(a.c0, rve, a.lam0, a.mu0, c1, c2h);
-    gc[0] = c1 * a.scale;
-    gc[1] = c2h * a.scale;
-  }
+  if (MODE != CGF_INIT) green_consts_shared<float>(gc, a.c0, rve, a.lam0, a.mu0);
+  else if (tid == 0) gc[0] = 1.0f, gc[1] = 0.5f;
   grid_dep_wait();
   const int active = a.st[rhs].active;
   fetch(blockIdx.x, 0);   // with the state on its way: a launch rarely holds loads that have ended
@@ -368,7 +364,7 @@ __global__ void __launch_bounds__(ZLaunch<N, TC>::threads, ZLaunch<N, TC>::min_b
   const float alpha = MODE == CGF_STEP ? (float)a.st[rhs].alpha : 0.0f;
   double sum_n = 0.0, sum_d = 0.0;   // weighted sums of |q|^2 |v|^2 and |q . v|^2 over the new r
   __syncthreads();   // tables
-  const float c1 = gc[0], c2h = gc[1];
+  const float c1 = gc[0] * a.scale, c2h = gc[1] * a.scale;
 #pragma unroll 1
   for (int tile = blockIdx.x; tile < ntiles; tile += step) {
     const unsigned f = (unsigned)tile * TC + tc;

@@ -19,7 +19,7 @@ namespace hom {
 // in it: on this GPU the FP64 pipe executes a small fraction of the FP32 rate, and these passes
 // need about 1e-12 relative accuracy, not 53 bits.  Sums use Knuth's TwoSum and Dekker's
 // FastTwoSum, products an FMA-exact product (the standard error-free transformations); the
-// division goes through double and is used once per frequency only.
+// division starts from the FP32 reciprocal.
 struct df64 {
   float hi, lo;
   df64() = default;
@@ -51,12 +51,40 @@ __device__ __forceinline__ df64 operator*(df64 a, df64 b) {
   e = __fmaf_rn(a.lo, b.hi, e);
   return df_fast_two_sum(p, e);
 }
-__device__ __forceinline__ df64 operator/(df64 a, df64 b) { return df64((double)a / (double)b); }
+// a / b from the FP32 reciprocal of b.hi: one Newton step in double-float, the quotient, and its remainder's
+// correction (no FP64: a warp instruction takes 16 cycles of that pipe, a division some 20 of them)
+__device__ __forceinline__ df64 operator/(df64 a, df64 b) {
+  const float r0 = 1.0f / b.hi;
+  const df64 r = df64(r0) + (df64(1.0f) - b * df64(r0)) * df64(r0);
+  const df64 q = a * r, rem = a - b * q;
+  return q + df64(rem.hi * r0);
+}
 __device__ __forceinline__ df64& operator+=(df64& a, df64 b) { return a = a + b; }
 __device__ __forceinline__ df64& operator-=(df64& a, df64 b) { return a = a - b; }
 __device__ __forceinline__ df64& operator*=(df64& a, df64 b) { return a = a * b; }
 __device__ __forceinline__ bool operator==(df64 a, df64 b) { return a.hi == b.hi && a.lo == b.lo; }
 __device__ __forceinline__ bool operator!=(df64 a, df64 b) { return !(a == b); }
+
+// A double as a double-float: hi rounded to nearest, lo the rest, by integer arithmetic on the bits (the
+// conversions and the subtraction of (float)(d - (double)(float)d) are FP64-pipe instructions, 16 cycles
+// per warp each, and these kernels read whole FP64 fields).  Values whose lo would leave the normal FP32
+// range, and infinities and NaN, take the conversions.
+__device__ __forceinline__ df64 df_from_double(double d) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(d), a = u & 0x7fffffffffffffffull;
+  const unsigned e = (unsigned)(a >> 52);
+  if (a == 0ull) return df64(__uint_as_float((unsigned)(u >> 32)), 0.0f);
+  if (e < 950u || e > 1148u) return df64(d);
+  const unsigned s = (unsigned)(u >> 32) & 0x80000000u;
+  const unsigned hi = (unsigned)((a + (1ull << 28)) >> 29) - (896u << 23);
+  int lo = (int)((unsigned)a & 0x1fffffffu);
+  if (lo & (1 << 28)) lo -= 1 << 29;
+  const float l = (float)lo * __uint_as_float((e - 948u) << 23);   // units of 2^(e - 1023 - 52)
+  return df64(__uint_as_float(hi | s), s ? -l : l);
+}
+// a field value in the compute type T
+template <typename T> __device__ __forceinline__ T to_compute(double d) { return (T)d; }
+template <> __device__ __forceinline__ df64 to_compute<df64>(double d) { return df_from_double(d); }
+template <typename T> __device__ __forceinline__ T to_compute(float f) { return (T)f; }
 
 template <typename T>
 struct alignas(2 * sizeof(T)) cx {

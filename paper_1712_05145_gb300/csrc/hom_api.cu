@@ -655,9 +655,6 @@ CgPass cg_pass(hom_ctx* c, cx<float>* rh, cx<float>* ph, cx<float>* xh) {
   za.rve_loads = c->rve_loads;
   za.c0 = c->rve_loads > 0 ? c->d_c0 : nullptr;
   za.scale = (float)(1.0 / (double)c->g.M);
-  za.xs[0] = (float)c->g.xs1;
-  za.xs[1] = (float)c->g.xs2;
-  za.xs[2] = (float)c->g.xs3;
   za.green = c->opt.green_operator;
   za.gtab = c->d_gtab;
   za.tw_n3 = tw<float>(c, 3);
@@ -2193,10 +2190,7 @@ HOM_API hom_status hom_create(const int32_t grid[3], const uint8_t* phase, int32
   g.plane_c = (long long)n2 * (g.h + 1);
   geo_finish(g);
   g.split = (pass_mode >= 2 || (pass_mode == 0 && (long long)g.n2 * g.h > 8192)) ? 1 : 0;
-  const int nmax = std::max(n1, std::max(n2, n3));
-  g.xs1 = 2.0 * M_PI * nmax / n1;
-  g.xs2 = 2.0 * M_PI * nmax / n2;
-  g.xs3 = 2.0 * M_PI * nmax / n3;
+  geo_wave_scale(g);
 
   auto bail = [&](hom_status s) {
     hom_destroy(c);

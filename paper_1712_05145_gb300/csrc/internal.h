@@ -27,6 +27,7 @@ struct Geo {
   int ty_log2, thr_y;    // y pass: 2^ty_log2 consecutive columns per CTA, threads
   FastDiv fd_ty;         // division by 2^ty_log2
   double xs1, xs2, xs3;  // physical frequency per integer wave number: 2 pi Nmax / N_i
+  df64 xsd[3];           // the same split in two floats
   // cluster plane passes (split grids, FP32 transforms): pc_Q CTAs per plane (0: not used), each
   // with pc_R = n2 / pc_Q rows and pc_Cb = h / pc_Q spectrum columns, pc_thr threads
   int pc_Q, pc_R, pc_Cb, pc_thr;
@@ -193,6 +194,8 @@ size_t plane_smem_bytes(const Geo& g, size_t elem);
 size_t zpass_smem_bytes(const Geo& g, size_t elem, int ncomp, int tc_log2);
 // fills fd_h, fd_n2 and the split-pass tiling of a geometry whose n1, n2, n3 are set
 void geo_finish(Geo& g);
+// the wave number scale of axes n1, n2, n3 (xs1 .. xsd)
+void geo_wave_scale(Geo& g);
 // y pass tiles of 2^lg columns (ty_log2, thr_y, fd_ty); whether such tiles fit the y pass
 void set_ytile(Geo& g, int lg);
 bool ytile_fits(const Geo& g, int lg);

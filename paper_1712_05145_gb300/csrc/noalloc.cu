@@ -129,10 +129,7 @@ HOM_API hom_status hom_ls_apply_noalloc(const int32_t grid[3], const uint8_t* ph
   g.M = (long long)n1 * n2 * n3;
   g.plane_c = (long long)n2 * (g.h + 1);
   geo_finish(g);
-  const int nmax = n1 > n2 ? (n1 > n3 ? n1 : n3) : (n2 > n3 ? n2 : n3);
-  g.xs1 = 2.0 * M_PI * nmax / n1;
-  g.xs2 = 2.0 * M_PI * nmax / n2;
-  g.xs3 = 2.0 * M_PI * nmax / n3;
+  geo_wave_scale(g);
 
   // carve the scratch: spectrum | twiddles (h, n1, n2, n3) | eigenvalues | loads
   size_t off = 0;

@@ -1,4 +1,6 @@
 // Forward plane pass of the Lippmann-Schwinger step (see ls_common.cuh).
+#include <cmath>
+
 #include "ls_common.cuh"
 
 namespace hom {
@@ -85,13 +87,13 @@ plane_fwd_kernel(const FwdArgs<Tf, T> a) {
         Tf v0 = 0, v1 = 0;
         if (a.in != nullptr) ld2<Tf>(a.in + foff + o, v0, v1);
         const uchar2 ph = *reinterpret_cast<const uchar2*>(php + o);
-        T t0 = w[ph.x] * ((T)v0 + ec), t1 = w[ph.y] * ((T)v1 + ec);
+        T t0 = w[ph.x] * (to_compute<T>(v0) + ec), t1 = w[ph.y] * (to_compute<T>(v1) + ec);
         if constexpr (std::is_same<T, df64>::value) {
           if (a.bsub != nullptr) {
             double b0, b1;
             ld2<double>(a.bsub + foff + o, b0, b1);
-            t0 -= wb * (T)b0;
-            t1 -= wb * (T)b1;
+            t0 -= wb * to_compute<T>(b0);
+            t1 -= wb * to_compute<T>(b1);
           }
         }
         pl[row * P + c2] = mk<T>(t0, t1);
@@ -155,7 +157,7 @@ plane_fwd_kernel(const FwdArgs<Tf, T> a) {
         const long long o = (long long)row * n1 + 2 * c2;
         Tf v0, v1;
         ld2<Tf>(a.in + foff + o, v0, v1);
-        pl[row * P + c2] = mk<T>(w * (T)v0, w * (T)v1);
+        pl[row * P + c2] = mk<T>(w * to_compute<T>(v0), w * to_compute<T>(v1));
       }
     }
   }
@@ -252,6 +254,16 @@ void geo_finish(Geo& g) {
   int lg = 0;
   while (lg < 4 && (g.h % (2 << lg)) == 0 && (long long)g.n2 * (2 << lg) <= (long long)kEPT * 512) ++lg;
   set_ytile(g, lg);
+}
+
+void geo_wave_scale(Geo& g) {
+  const int m = g.n2 > g.n3 ? g.n2 : g.n3, nmax = g.n1 > m ? g.n1 : m;
+  g.xs1 = 2.0 * M_PI * nmax / g.n1;
+  g.xs2 = 2.0 * M_PI * nmax / g.n2;
+  g.xs3 = 2.0 * M_PI * nmax / g.n3;
+  g.xsd[0] = df64(g.xs1);
+  g.xsd[1] = df64(g.xs2);
+  g.xsd[2] = df64(g.xs3);
 }
 
 bool ytile_fits(const Geo& g, int lg) {

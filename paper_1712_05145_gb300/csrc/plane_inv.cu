@@ -126,8 +126,8 @@ plane_inv_kernel(const InvArgs<Tf, T> a) {
         const long long o = foff + (long long)row * n1 + 2 * c2;
         const cx<T> e = pl[row * P + c2];
         T v0 = a.out_scale * e.re, v1 = a.out_scale * e.im;
-        if (a.b != nullptr) { double b0, b1; ld2<double>(a.b + o, b0, b1); v0 += (T)b0; v1 += (T)b1; }
-        if (a.xsub != nullptr) { double s0, s1; ld2<double>(a.xsub + o, s0, s1); v0 -= (T)s0; v1 -= (T)s1; }
+        if (a.b != nullptr) { double b0, b1; ld2<double>(a.b + o, b0, b1); v0 += to_compute<T>(b0); v1 += to_compute<T>(b1); }
+        if (a.xsub != nullptr) { double s0, s1; ld2<double>(a.xsub + o, s0, s1); v0 -= to_compute<T>(s0); v1 -= to_compute<T>(s1); }
         if (a.fin == FIN_BASIC) {
           Tf p0, p1;
           ld2<Tf>(a.prev + o, p0, p1);

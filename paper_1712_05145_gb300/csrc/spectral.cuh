@@ -2,7 +2,7 @@
 // check: the Kelvin basis of symmetric tensors, the product with a wave vector, and the
 // discrete wave numbers of the half spectrum.
 #pragma once
-#include "common.cuh"
+#include "internal.h"
 
 namespace hom {
 
@@ -45,6 +45,31 @@ __device__ __forceinline__ void green_consts(const double* c0, int rve, double l
   c2h = (T)((lam0 + mu0) / (2.0 * mu0 * (lam0 + 2.0 * mu0)));
 }
 
+// The same by the CTA's thread 0 into shared memory (dst[2]); a barrier follows in the caller.  (In every
+// thread, the two FP64 divisions kept the FP32 z passes waiting for the FP64 pipe.)
+template <typename T>
+__device__ __forceinline__ void green_consts_shared(T* dst, const double* c0, int rve, double lam0, double mu0) {
+  if (threadIdx.x == 0) {
+    T c1, c2h;
+    green_consts<T>(c0, rve, lam0, mu0, c1, c2h);
+    dst[0] = c1;
+    dst[1] = c2h;
+  }
+}
+
+// physical frequency of the integer wave number k on axis i: k xs, rounded once; without the FP64 pipe in
+// FP32 and double-float (k is exact in FP32)
+template <typename T> __device__ __forceinline__ T wave_scaled(const Geo& g, int i, int k) {
+  return (T)(k * (i == 0 ? g.xs1 : i == 1 ? g.xs2 : g.xs3));
+}
+template <> __device__ __forceinline__ float wave_scaled<float>(const Geo& g, int i, int k) {
+  const float f = (float)k;
+  return fmaf(f, g.xsd[i].hi, f * g.xsd[i].lo);
+}
+template <> __device__ __forceinline__ df64 wave_scaled<df64>(const Geo& g, int i, int k) {
+  return df64((float)k) * g.xsd[i];
+}
+
 // The vector at which Gamma0_hat is evaluated for the half-spectrum frequency (kx, ky, n):
 //  green == 0: the discrete wave vector xi (Nyquist components 0);
 //  green == 1: the rotated finite-difference symbol q_j = sin(xi_j h/2) prod_{l != j} cos(xi_l h/2)
@@ -55,9 +80,9 @@ template <typename T>
 __device__ __forceinline__ void wave_vector(const Geo& g, int green, const double* gtab, int kx, int ky, int n,
                                             T& x1, T& x2, T& x3) {
   if (green == 0) {
-    x1 = (T)((kx == g.h ? 0 : kx) * g.xs1);
-    x2 = (T)(wave(ky, g.n2) * g.xs2);
-    x3 = (T)(wave(n, g.n3) * g.xs3);
+    x1 = wave_scaled<T>(g, 0, kx == g.h ? 0 : kx);
+    x2 = wave_scaled<T>(g, 1, wave(ky, g.n2));
+    x3 = wave_scaled<T>(g, 2, wave(n, g.n3));
   } else {
     const double* t2 = gtab + 2 * (g.h + 1);
     const double* t3 = t2 + 2 * g.n2;

@@ -147,20 +147,20 @@ __global__ void __launch_bounds__(256 * (kEPT / EPT), XfCfg<T>::kMinBlocks) xpas
             Tf v0 = 0, v1 = 0;
             if (a.in != nullptr) ld2<Tf>(a.in + cbase + o, v0, v1);
             const uchar2 ph = *reinterpret_cast<const uchar2*>(phase + o);
-            val = mk<T>(w[ph.x] * ((T)v0 + ec), w[ph.y] * ((T)v1 + ec));
+            val = mk<T>(w[ph.x] * (to_compute<T>(v0) + ec), w[ph.y] * (to_compute<T>(v1) + ec));
             if constexpr (std::is_same<T, df64>::value) {
               if (a.bsub != nullptr) {
                 const T wb = (c == 0) ? ch : cd;
                 double b0, b1;
                 ld2<double>(a.bsub + cbase + o, b0, b1);
-                val.re -= wb * (T)b0;
-                val.im -= wb * (T)b1;
+                val.re -= wb * to_compute<T>(b0);
+                val.im -= wb * to_compute<T>(b1);
               }
             }
           } else {
             Tf v0, v1;
             ld2<Tf>(a.in + cbase + o, v0, v1);
-            val = mk<T>(wc * (T)v0, wc * (T)v1);
+            val = mk<T>(wc * to_compute<T>(v0), wc * to_compute<T>(v1));
           }
         }
         pl[lr * P + c2] = val;
@@ -325,8 +325,8 @@ __global__ void __launch_bounds__(256 * (kEPT / EPT), std::is_same<T, df64>::val
         const long long o = cbase + (r0 + lr) * n1 + 2 * c2;
         const cx<T> e = pl[lr * P + c2];
         T v0 = a.out_scale * e.re, v1 = a.out_scale * e.im;
-        if (a.b != nullptr) { double b0, b1; ld2<double>(a.b + o, b0, b1); v0 += (T)b0; v1 += (T)b1; }
-        if (a.xsub != nullptr) { double s0, s1; ld2<double>(a.xsub + o, s0, s1); v0 -= (T)s0; v1 -= (T)s1; }
+        if (a.b != nullptr) { double b0, b1; ld2<double>(a.b + o, b0, b1); v0 += to_compute<T>(b0); v1 += to_compute<T>(b1); }
+        if (a.xsub != nullptr) { double s0, s1; ld2<double>(a.xsub + o, s0, s1); v0 -= to_compute<T>(s0); v1 -= to_compute<T>(s1); }
         if (a.fin == FIN_BASIC) {
           Tf p0, p1;
           ld2<Tf>(a.prev + o, p0, p1);

@@ -80,6 +80,8 @@ __global__ void __cluster_dims__(kZcComps, 1, 1) __launch_bounds__(ZcCfg<T>::kTh
     atomicAdd(a.prof, (unsigned long long)(2LL * n3 * cols * (long long)sizeof(cx<T>)));
     if (comp == 0) atomicAdd(a.prof + 1, (unsigned long long)(n3 * cols));
   }
+  __shared__ T gc[2];
+  green_consts_shared<T>(gc, a.c0, rve_of(rhs, a.rve_loads), a.lam0, a.mu0);
   cp_async_wait_all();
   __syncthreads();
   fft_pencils<T, -1, EPT>(buf, ColAddr{TC}, n3, TC, a.fd_in, twz);
@@ -89,8 +91,7 @@ __global__ void __cluster_dims__(kZcComps, 1, 1) __launch_bounds__(ZcCfg<T>::kTh
     cx<T>* part[kZcComps];
 #pragma unroll
     for (int r = 0; r < kZcComps; ++r) part[r] = cl.map_shared_rank(buf, r);
-    T c1, c2h;
-    green_consts<T>(a.c0, rve_of(rhs, a.rve_loads), a.lam0, a.mu0, c1, c2h);
+    const T c1 = gc[0], c2h = gc[1];
     const T scale = (T)a.scale;
     const long long nmain = (long long)g.n2 * g.h;
     const int share = (per + kZcComps - 1) / kZcComps;
@@ -153,6 +154,9 @@ __global__ void __cluster_dims__(kZcComps, 1, 1) __launch_bounds__(512, 2)
     mbar_arrive_expect_tx(bar, (uint32_t)nbox * box_bytes);
     for (int b = 0; b < nbox; ++b) tma_load_3d(sbuf + b * box_bytes, &tm, tile * TC, b * rows, zc, bar);
   }
+  // after the mbarrier, not in static shared memory, which would move the tile off its 128-byte boundary
+  float* gc = reinterpret_cast<float*>(twz + n3) + 2;
+  green_consts_shared<float>(gc, a.c0, rve_of(rhs, a.rve_loads), a.lam0, a.mu0);
   for (int i = tid; i < n3; i += blockDim.x) twz[i] = ldg_cx(a.tw_n3 + i);
   __syncthreads();   // the mbarrier is initialised before anyone waits on it
   const bool ok = mbar_wait_bounded(bar, 0, kZtWaitNs);
@@ -162,8 +166,7 @@ __global__ void __cluster_dims__(kZcComps, 1, 1) __launch_bounds__(512, 2)
     cx<float>* part[kZcComps];
 #pragma unroll
     for (int r = 0; r < kZcComps; ++r) part[r] = cl.map_shared_rank(buf, r);
-    float c1, c2h;
-    green_consts<float>(a.c0, rve_of(rhs, a.rve_loads), a.lam0, a.mu0, c1, c2h);
+    const float c1 = gc[0], c2h = gc[1];
     const float scale = (float)a.scale;
     const long long nmain = (long long)g.n2 * g.h, f0 = (long long)tile * TC;
     const int share = (per + kZcComps - 1) / kZcComps;

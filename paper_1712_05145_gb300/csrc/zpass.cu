@@ -13,8 +13,10 @@ namespace hom {
 template <typename T>
 __global__ void __launch_bounds__(256) zgreen_kernel(const ZArgs<T> a, int nrhs) {
   const Geo& g = a.g;
-  T c1, c2h;
-  green_consts<T>(nullptr, 0, a.lam0, a.mu0, c1, c2h);
+  __shared__ T gc[2];
+  green_consts_shared<T>(gc, nullptr, 0, a.lam0, a.mu0);
+  __syncthreads();
+  T c1 = gc[0], c2h = gc[1];
   const T scale = (T)a.scale;
   const long long per = (long long)g.n3 * g.plane_c;   // frequencies of one component
   const long long nmain = (long long)g.n2 * g.h;
@@ -83,6 +85,8 @@ __global__ void __launch_bounds__(512) zpass_kernel(const ZArgs<T> a) {
     atomicAdd(a.prof + 1, (unsigned long long)(n3 * cols));
   }
 
+  __shared__ T gc[2];
+  green_consts_shared<T>(gc, a.c0, rve_of(rhs, a.rve_loads), a.lam0, a.mu0);
   const int per_c = n3 * TC;
   {
     // the whole tile is in flight at once: cp.async per element, zeros past the last column
@@ -101,8 +105,7 @@ __global__ void __launch_bounds__(512) zpass_kernel(const ZArgs<T> a) {
   if (a.mode != Z_INV && a.mode != Z_GREEN) fft_pencils<T, -1, EPT>(buf, za, n3, a.ncomp_in * TC, a.fd_in, twz);
 
   if (a.mode == Z_GAMMA || a.mode == Z_GREEN || a.mode == Z_DISP || a.mode == Z_RHS) {
-    T c1, c2h;
-    green_consts<T>(a.c0, rve_of(rhs, a.rve_loads), a.lam0, a.mu0, c1, c2h);
+    const T c1 = gc[0], c2h = gc[1];
     const T scale = (T)a.scale;
     const long long nmain = (long long)g.n2 * g.h;
     for (int t = tid; t < n3 * TC; t += nthr) {
