@@ -1,7 +1,7 @@
 // BiCGSTAB on the Lippmann-Schwinger system A eps = b (Eq. cg_form), the Krylov solver the paper
 // ran for its CG-version (Sec. 4).  The two operator applications per iteration, v = A p and
 // t = A s, are LS passes (A = Gamma0 * (C : .) on compatible fields); this file holds the vector
-// updates between them.  Each step is one grid-stride kernel over the [6][M] field of every
+// updates between them on real FP64 fields (FP32 BiCGSTAB runs in Fourier space, cg_bicg.cu).  Each step is one grid-stride kernel over the [6][M] field of every
 // active load, with FP64 block sums and a last-block ticket that updates the load's state:
 //   BI_RESTART  r_hat = r, p = r                      rho = <r, r>
 //   BI_ALPHA    (reads v = A p)                       alpha = rho / <r_hat, v>
@@ -15,60 +15,6 @@
 #include "ls_common.cuh"
 
 namespace hom {
-
-__device__ __forceinline__ void bicg_finalize(int step, RhsState& s, const double* v, double invM) {
-  switch (step) {
-    case BI_RESTART: {
-      s.rho = v[0] * invM;
-      s.rr = s.rho;
-      s.restart = 0;
-      s.sconv = 0;
-      if (!isfinite(s.rho)) { s.status = 2; s.active = 0; }
-      break;
-    }
-    case BI_ALPHA: {
-      const double rv = v[0] * invM;
-      s.alpha = (rv != 0.0) ? s.rho / rv : 0.0;
-      s.sconv = 0;
-      if (!isfinite(s.alpha)) { s.status = 2; s.active = 0; }
-      break;
-    }
-    case BI_S: {
-      const double ss = v[0] * invM;
-      s.sconv = (s.b2 > 0.0 && sqrt(ss / s.b2) < s.tol) ? 1 : 0;
-      break;
-    }
-    case BI_OMEGA: {
-      const double ts = v[0] * invM, tt = v[1] * invM;
-      s.omega = (s.sconv || tt <= 0.0) ? 0.0 : ts / tt;
-      if (!isfinite(s.omega)) { s.status = 2; s.active = 0; }
-      break;
-    }
-    case BI_X: {
-      const double rho = v[0] * invM, rr = v[1] * invM;
-      s.rr = rr;
-      s.res = (s.b2 > 0.0) ? sqrt(rr / s.b2) : 0.0;
-      s.iter += 1;
-      if (s.omega != 0.0 && rho != 0.0 && s.rho != 0.0) {
-        s.beta = (rho / s.rho) * (s.alpha / s.omega);
-        s.rho = rho;
-        s.restart = 0;
-      } else {  // breakdown: restart from r_hat = r
-        s.beta = 0.0;
-        s.rho = rr;
-        s.restart = 1;
-      }
-      if (!isfinite(s.res) || !isfinite(s.beta)) { s.status = 2; s.active = 0; }
-      else if (s.res < s.tol) s.active = 0;
-      else if (s.iter >= s.max_iter) { s.active = 0; s.status = 1; }
-      else if (s.res < 0.5 * s.best) { s.best = s.res; s.best_iter = s.iter; }
-      else if (s.stall && s.iter - s.best_iter >= (s.res < kNearFloor ? kStallItersNearFloor : kStallIters))
-        s.active = 0;  // stalled: hand over to the FP64 residual sweep
-      break;
-    }
-    default: break;
-  }
-}
 
 template <typename Tf, int STEP>
 __global__ void __launch_bounds__(256) bicg_kernel(const BicgArgs<Tf> a) {
@@ -141,7 +87,6 @@ cudaError_t launch_bicg(int step, const BicgArgs<Tf>& a, int nrhs, int nblk, cud
   return cudaGetLastError();
 }
 
-template cudaError_t launch_bicg<float>(int, const BicgArgs<float>&, int, int, cudaStream_t);
 template cudaError_t launch_bicg<double>(int, const BicgArgs<double>&, int, int, cudaStream_t);
 
 }  // namespace hom

@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(512, 2) cg_plane_kernel(const CgPlaneArgs a) {
     atomicAdd(a.prof, (unsigned long long)(2 * g.plane_c * (long long)sizeof(cx<float>) + (long long)n2 * n1));
     atomicAdd(a.prof + 1, (unsigned long long)((long long)n2 * n1));
   }
-  if (tid < 32) {   // y_forward's barriers have made red complete
+  if (tid < 32 && a.fin == FIN_ENERGY) {   // y_forward's barriers have made red complete
     double v[1] = {2.0 * warp_sum_f64(m.red, nthr)};
     const int ncta = 6 * g.n3;
     if (warp_publish_and_collect<1>(v, a.part + (long long)rhs * 2 * ncta, a.cnt + rhs, ncta, c * g.n3 + z) && tid == 0)

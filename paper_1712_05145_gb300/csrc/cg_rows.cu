@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(kRowThreads, 4) cg_rows_kernel(const CgPlaneAr
     atomicAdd(a.prof, (unsigned long long)(2LL * nr * H * (long long)sizeof(cx<float>) + vox));
     atomicAdd(a.prof + 1, (unsigned long long)vox);
   }
-  if (tid < 32) {
+  if (tid < 32 && a.fin == FIN_ENERGY) {
     double v[1] = {2.0 * warp_sum_f64(red, kRowThreads)};
     const int ncta = 6 * gridDim.x;
     if (warp_publish_and_collect<1>(v, a.part + (long long)rhs * 2 * ncta, a.cnt + rhs, ncta,

@@ -664,6 +664,7 @@ CgPass cg_pass(hom_ctx* c, cx<float>* rh, cx<float>* ph, cx<float>* xh) {
   CgPlaneArgs& pa = q.pa;
   pa.g = c->g;
   pa.S = S;
+  pa.fin = FIN_ENERGY;
   pa.st = c->d_st;
   pa.phase = c->d_phase;
   pa.mat = c->d_mat32;
@@ -679,24 +680,45 @@ CgPass cg_pass(hom_ctx* c, cx<float>* rh, cx<float>* ph, cx<float>* xh) {
   return q;
 }
 
-// `iters` CG iterations of the m loads from r0 on (inactive loads are skipped on the device)
-hom_status cg_iterations(hom_ctx* c, CgPass& q, int r0, int m, int iters) {
+// The middle pass of m loads: inverse x-y transforms, tau = C : (.), forward transforms
+hom_status cg_middle(hom_ctx* c, const CgPass& q, int r0, int m) {
   unsigned long long* yp = c->prof_on ? c->d_prof + 2 * HOM_KERNEL_YPASS : nullptr;
   auto y = [&](int dir) {
     return timed_launch(c, HOM_KERNEL_YPASS,
                         [&] { return ypass<float>(c, q.pa.tw_n2, q.pa.S, 6, 6, m, dir, yp, c->d_st, r0); });
   };
+  if (q.whole_planes)
+    return timed_launch(c, HOM_KERNEL_PLANE_INV, [&] { return launch_cg_plane(q.pa, m, c->stream); });
+  CKS(y(+1));
+  CKS(timed_launch(c, HOM_KERNEL_PLANE_INV, [&] { return launch_cg_rows(q.pa, m, c->stream); }));
+  return y(-1);
+}
+
+// `iters` CG iterations of the m loads from r0 on (inactive loads are skipped on the device)
+hom_status cg_iterations(hom_ctx* c, CgPass& q, int r0, int m, int iters) {
   q.za.rhs0 = q.pa.rhs0 = r0;
   for (int k = 0; k < iters; ++k) {
     CKS(timed_launch(c, HOM_KERNEL_ZPASS, [&] { return launch_cg_z_inv(q.za, CGI_STEP, m, c->stream); }));
-    if (q.whole_planes) {
-      CKS(timed_launch(c, HOM_KERNEL_PLANE_INV, [&] { return launch_cg_plane(q.pa, m, c->stream); }));
-    } else {
-      CKS(y(+1));
-      CKS(timed_launch(c, HOM_KERNEL_PLANE_INV, [&] { return launch_cg_rows(q.pa, m, c->stream); }));
-      CKS(y(-1));
-    }
+    CKS(cg_middle(c, q, r0, m));
     CKS(timed_launch(c, HOM_KERNEL_ZPASS, [&] { return launch_cg_z_fwd(q.za, CGF_STEP, m, c->stream); }));
+  }
+  return HOM_OK;
+}
+
+// The same for BiCGSTAB (cg_bicg.cu), two operator applications per iteration
+hom_status bicg_iterations(hom_ctx* c, CgPass& q, int r0, int m, int iters) {
+  q.za.rhs0 = q.pa.rhs0 = r0;
+  auto z = [&](int step) {
+    return timed_launch(c, HOM_KERNEL_ZPASS, [&] { return launch_cg_bicg(q.za, step, m, c->stream); });
+  };
+  for (int k = 0; k < iters; ++k) {
+    CKS(z(BI_P));
+    CKS(cg_middle(c, q, r0, m));
+    CKS(z(BI_ALPHA));
+    CKS(z(BI_S));
+    CKS(cg_middle(c, q, r0, m));
+    CKS(z(BI_OMEGA));
+    CKS(z(BI_X));
   }
   return HOM_OK;
 }
@@ -763,8 +785,8 @@ hom_status cg_residual_fourier(hom_ctx* c, int n, const double* dE, const double
   return HOM_OK;
 }
 
-// One FP32 CG sweep on A d = r (Eq. cg_form) with its vectors in Fourier space, for the active loads:
-// r (real, compatible; nullptr if rh holds it already) goes to rh, CG runs until every load's device
+// One FP32 CG or BiCGSTAB sweep on A d = r (Eq. cg_form) with its vectors in Fourier space, for the
+// active loads: r (real, compatible; nullptr if rh holds it already) goes to rh, CG runs until every load's device
 // state is inactive, and the correction d is added to x64, through double-float transforms if df is
 // given.  rh, ph, xh: n loads' vectors (hat_bytes); ph may be r's buffer, which is read before the first
 // iteration writes p.  A chunk of loads runs check_every iterations before the next chunk starts, so
@@ -774,6 +796,27 @@ hom_status cg_sweep_fourier(hom_ctx* c, int n, const float* r, cx<float>* rh, cx
   const std::vector<int> ran = act;
   const int chunk = c->chunk;
   CgPass q = cg_pass(c, rh, ph, xh);
+  const bool bicg = c->opt.scheme == HOM_BICGSTAB;
+  if (bicg) {
+    const size_t hb = hat_bytes(c, n);
+    if (c->bicg_bytes < 4 * hb) {
+      if (c->d_bicg) dfree(c, c->d_bicg, c->bicg_bytes);
+      c->d_bicg = nullptr;
+      c->bicg_bytes = 0;
+      CKS(dalloc(c, &c->d_bicg, 4 * hb));
+      c->bicg_bytes = 4 * hb;
+    }
+    cx<float>** vec[4] = {&q.za.rh, &q.za.v, &q.za.s, &q.za.t};
+    for (int i = 0; i < 4; ++i) *vec[i] = reinterpret_cast<cx<float>*>(reinterpret_cast<char*>(c->d_bicg) + i * hb);
+    q.pa.fin = FIN_NONE;
+    // its inner products are L2; the first pass restarts from r_hat = r, p = r
+    for (auto& s : st) {
+      s.rho = s.b2 * s.res_true * s.res_true;
+      s.restart = 1;
+      s.sconv = 0;
+    }
+    CKS(write_states(c, st));
+  }
   // r -> rh
   auto fa = fwd_args<float, float>(c, FWD_COPY, 6, 6);
   fa.in = r;
@@ -791,7 +834,9 @@ hom_status cg_sweep_fourier(hom_ctx* c, int n, const float* r, cx<float>* rh, cx
   while (any) {
     for (int r0 = 0; r0 < n; r0 += chunk) {
       const int m = std::min(chunk, n - r0);
-      if (any_of(act, r0, m)) CKS(cg_iterations(c, q, r0, m, c->opt.check_every));
+      if (!any_of(act, r0, m)) continue;
+      if (bicg) CKS(bicg_iterations(c, q, r0, m, c->opt.check_every));
+      else CKS(cg_iterations(c, q, r0, m, c->opt.check_every));
     }
     CKS(read_states(c, n, st));
     any = false;
@@ -1063,8 +1108,7 @@ hom_status autotune(hom_ctx* c) {
   return HOM_OK;
 }
 
-// One BiCGSTAB sweep on A x = r from the current x (FP64 mode: the solution; FP32 mode: the
-// correction d), until every load's device state is inactive.
+// One FP64 BiCGSTAB sweep on A x = r from the current x, until every load's device state is inactive.
 template <typename Tf>
 hom_status bicgstab_sweep(hom_ctx* c, int n, Tf* x, Tf* r, Tf* p, std::vector<RhsState>& st, std::vector<int>& act) {
   const size_t fb = tbytes<Tf>(c, n, 6);
@@ -1248,7 +1292,8 @@ hom_status solve_system(hom_ctx* c, int n, const double* dE, const double* b64, 
                         hom_solve_info* info) {
   const bool mixed = sizeof(Tf) == sizeof(float);
   CKS(ensure_cap(c, n));
-  const bool fourier = mixed && c->opt.scheme == HOM_CG;   // FP32 CG keeps its vectors in Fourier space
+  // FP32 CG and BiCGSTAB keep their vectors in Fourier space
+  const bool fourier = mixed && (c->opt.scheme == HOM_CG || c->opt.scheme == HOM_BICGSTAB);
   const size_t fb = fourier ? std::max(tbytes<Tf>(c, n, 6), hat_bytes(c, n)) : tbytes<Tf>(c, n, 6);
   void *vr, *vp, *vd = nullptr;
   CKS(work(c, 0, fb, &vr));
@@ -1266,9 +1311,9 @@ hom_status solve_system(hom_ctx* c, int n, const double* dE, const double* b64, 
   // the FP64 residual they restart from.
   const double kSweepGain = 1e-5, kFirstSweepTarget = 1e-4, kFp32OutTol = 5e-7;
   const double tol_inner = (mixed && !basic) ? std::max(0.5 * tol, kFirstSweepTarget) : (mixed ? 0.5 * tol : tol);
-  // FP32 corrections computed on real fields (BiCGSTAB) leave an incompatible part in x: step lengths
-  // reach C0 / C_min along the soft phases' directions and multiply the FP32 rounding of each direction
-  // p by as much (4.4e-5 of ||b|| at 128^3 and contrast 100).  The residual form b - Gamma0 * (C : x)
+  // FP32 corrections computed on real fields (the polarization scheme's; CG's once were) leave an
+  // incompatible part in x, multiplied by the stiffness contrast (CG: 4.4e-5 of ||b|| at 128^3 and
+  // contrast 100).  The residual form b - Gamma0 * (C : x)
   // does not see it, but the operator of Eq. cg_form does.  So in FP32 mode:
   //  * a sweep that aimed at the tolerance is verified with the literal residual b - A x (one
   //    FP64 pass, which sees the incompatible part); below tol the load is done;
@@ -1276,7 +1321,7 @@ hom_status solve_system(hom_ctx* c, int n, const double* dE, const double* b64, 
   //    the projected x (two FP64 passes).  The first sweep aims only at kFirstSweepTarget: the
   //    projection after it perturbs the residual by about the incompatible part anyway, and the
   //    later sweeps, whose corrections are small, leave a negligible incompatible part.
-  // FP32 CG keeps its vectors in Fourier space, where they are compatible by construction; what its
+  // FP32 CG and BiCGSTAB keep their vectors in Fourier space, where they are compatible by construction; what its
   // correction adds to x is incompatible by the rounding of one FP32 transform, no more than the
   // FP32 projection left, so its first restart needs none.
   // The polarization scheme's iterates are compatible only at the fixed point, so it takes the
@@ -1411,9 +1456,11 @@ hom_status solve_system(hom_ctx* c, int n, const double* dE, const double* b64, 
     for (int sweep = 0;; ++sweep) {
       bool any = false;
       for (int i = 0; i < n; ++i) any = any || act[i];
-      if (bicg && any) {
-        CKS(bicgstab_sweep<Tf>(c, n, d, r, p, st, act));
-        any = false;
+      if constexpr (std::is_same<Tf, double>::value) {
+        if (bicg && any) {
+          CKS(bicgstab_sweep<Tf>(c, n, d, r, p, st, act));
+          any = false;
+        }
       }
       if (polar && any) {
         CKS(polar_sweep<Tf>(c, n, d, r, p, st, act));
@@ -1537,7 +1584,9 @@ hom_status solve_system(hom_ctx* c, int n, const double* dE, const double* b64, 
         } else if (refine[i] < c->opt.max_refine && st[i].iter < st[i].max_iter) {
           refine[i] += 1;
           st[i].active = 1;  // restart CG from the FP64 residual
-          st[i].tol = mixed ? std::max(0.5 * tol, kSweepGain * st[i].res_true) : 0.5 * tol;
+          // (a BiCGSTAB step reduces the residual by several times: one that ends just below half the
+          // tolerance leaves up to twice the error of one that ends well below, for the same count)
+          st[i].tol = mixed ? std::max((bicg ? 0.25 : 0.5) * tol, kSweepGain * st[i].res_true) : 0.5 * tol;
           st[i].best = 1e300;
           st[i].best_iter = st[i].iter;
           again = true;

@@ -263,6 +263,61 @@ __device__ __forceinline__ void finalize_state(int kind, RhsState& s, const doub
   }
 }
 
+// BiCGSTAB state updates (bicgstab.cu, cg_bicg.cu)
+__device__ __forceinline__ void bicg_finalize(int step, RhsState& s, const double* v, double invM) {
+  switch (step) {
+    case BI_RESTART: {
+      s.rho = v[0] * invM;
+      s.rr = s.rho;
+      s.restart = 0;
+      s.sconv = 0;
+      if (!isfinite(s.rho)) { s.status = 2; s.active = 0; }
+      break;
+    }
+    case BI_ALPHA: {
+      const double rv = v[0] * invM;
+      s.alpha = (rv != 0.0) ? s.rho / rv : 0.0;
+      s.sconv = 0;
+      if (!isfinite(s.alpha)) { s.status = 2; s.active = 0; }
+      break;
+    }
+    case BI_S: {
+      const double ss = v[0] * invM;
+      s.sconv = (s.b2 > 0.0 && sqrt(ss / s.b2) < s.tol) ? 1 : 0;
+      break;
+    }
+    case BI_OMEGA: {
+      const double ts = v[0] * invM, tt = v[1] * invM;
+      s.omega = (s.sconv || tt <= 0.0) ? 0.0 : ts / tt;
+      if (!isfinite(s.omega)) { s.status = 2; s.active = 0; }
+      break;
+    }
+    case BI_X: {
+      const double rho = v[0] * invM, rr = v[1] * invM;
+      s.rr = rr;
+      s.res = (s.b2 > 0.0) ? sqrt(rr / s.b2) : 0.0;
+      s.iter += 1;
+      if (s.omega != 0.0 && rho != 0.0 && s.rho != 0.0) {
+        s.beta = (rho / s.rho) * (s.alpha / s.omega);
+        s.rho = rho;
+        s.restart = 0;
+      } else {  // breakdown: restart from r_hat = r
+        s.beta = 0.0;
+        s.rho = rr;
+        s.restart = 1;
+      }
+      if (!isfinite(s.res) || !isfinite(s.beta)) { s.status = 2; s.active = 0; }
+      else if (s.res < s.tol) s.active = 0;
+      else if (s.iter >= s.max_iter) { s.active = 0; s.status = 1; }
+      else if (s.res < 0.5 * s.best) { s.best = s.res; s.best_iter = s.iter; }
+      else if (s.stall && s.iter - s.best_iter >= (s.res < kNearFloor ? kStallItersNearFloor : kStallIters))
+        s.active = 0;  // stalled: hand over to the FP64 residual sweep
+      break;
+    }
+    default: break;
+  }
+}
+
 // Dynamic shared memory above 48 KB needs an opt-in; the carveout asks for the largest shared
 // memory partition so that the occupancy is not limited by a small default carveout.  The
 // opt-in is a per-function, per-context limit shared by every host thread, so it is always set

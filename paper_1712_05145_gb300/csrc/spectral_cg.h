@@ -21,6 +21,7 @@ struct CgZArgs {
   cx<float>* r;            // [rhs][tile of columns][3][n3][columns] each (cg_vector_elems per rhs)
   cx<float>* p;
   cx<float>* x;
+  cx<float>*rh, *v, *s, *t;  // BiCGSTAB: r_hat, v = A p, s, t = A s
   int rhs0;
   RhsState* st;
   double lam0, mu0;
@@ -38,8 +39,9 @@ struct CgZArgs {
 // cg_z_inv: CGI_STEP the iteration's first pass; CGI_OUT x += alpha p where pending, strain of x -> S
 // cg_z_fwd: CGF_STEP the iteration's last pass; CGF_INIT r = the components v of a compatible strain;
 //           CGF_RHS r = -Gamma0_hat : tau_hat with its norms (the right-hand side, from tau = (C - C0) : E)
-enum CgInvMode { CGI_STEP = 0, CGI_OUT = 1 };
-enum CgFwdMode { CGF_STEP = 0, CGF_INIT = 1, CGF_RHS = 2 };
+// The BI modes are BiCGSTAB's (cg_bicg.cu).
+enum CgInvMode { CGI_STEP = 0, CGI_OUT = 1, CGI_BI_P = 2, CGI_BI_S = 3 };
+enum CgFwdMode { CGF_STEP = 0, CGF_INIT = 1, CGF_RHS = 2, CGF_BI_V = 3, CGF_BI_T = 4 };
 
 // z passes in double-float around a sweep (cg_df.cu), with the tiles of the cluster z pass
 struct CgDfArgs {
@@ -74,6 +76,7 @@ cudaError_t launch_cg_df_out(const CgDfArgs& a, int nrhs, cudaStream_t s);
 struct CgPlaneArgs {
   Geo g;
   cx<float>* S;
+  int fin;                 // FIN_ENERGY: reduce <p, C p>; FIN_NONE (BiCGSTAB)
   int rhs0;
   RhsState* st;
   const uint8_t* phase;    // [rve][n3][n2][n1]
@@ -93,6 +96,8 @@ int cg_vector_tile(const Geo& g);         // columns of one of its tiles (a powe
 int cg_z_blocks(const Geo& g);            // CTAs of one load in the z passes
 cudaError_t launch_cg_z_inv(const CgZArgs& a, int mode, int nrhs, cudaStream_t s);
 cudaError_t launch_cg_z_fwd(const CgZArgs& a, int mode, int nrhs, cudaStream_t s);
+// one of BiCGSTAB's passes (BI_P, BI_ALPHA, BI_S, BI_OMEGA, BI_X; cg_bicg.cu)
+cudaError_t launch_cg_bicg(const CgZArgs& a, int step, int nrhs, cudaStream_t s);
 // whether one CTA holds a plane of the grid in cg_plane (else the y pass and cg_rows run)
 bool cg_plane_fits(const Geo& g);
 cudaError_t launch_cg_plane(const CgPlaneArgs& a, int nrhs, cudaStream_t s);

@@ -1,4 +1,4 @@
-"""FP32 CG with its vectors in Fourier space against the FP64 mode's CG on real fields, at every axis
+"""FP32 CG and BiCGSTAB with their vectors in Fourier space against the FP64 mode's CG on real fields, at every axis
 length of the z, y and row transforms, through whole planes and through rows and columns.
 
 Tolerance.  The phases' moduli lie between 0.106 and 2 times the reference medium's (3 lambda + 2 mu =
@@ -24,15 +24,13 @@ def _ms(grid, seed):
     return synthetic.Microstructure(random_phase(grid, 3, seed, p=[0.5, 0.3, 0.2]), LAME, 4.0, 2.5)
 
 
-@pytest.mark.parametrize("pass_mode", [0, 2])
-@pytest.mark.parametrize("grid", GRIDS, ids=["x".join(map(str, g)) for g in GRIDS])
-def test_fp32_cg_matches_fp64_cg(grid, pass_mode):
+def _compare(grid, pass_mode, scheme32):
     from paper_1712_05145_gb300 import hom
     ms = _ms(grid, sum(grid))
     loads = np.eye(6)[[0, 5]] + 0.25 * np.eye(6)[[1, 3]]
     got = []
-    for precision, tol in ((hom.HOM_FP32_REFINE, 1e-6), (hom.HOM_FP64, 1e-10)):
-        H = hom.Homogenization(ms, precision=precision, pass_mode=pass_mode)
+    for precision, scheme, tol in ((hom.HOM_FP32_REFINE, scheme32, 1e-6), (hom.HOM_FP64, hom.HOM_CG, 1e-10)):
+        H = hom.Homogenization(ms, precision=precision, scheme=scheme, pass_mode=pass_mode)
         info = H.solve(0, tol, loads=loads)
         assert all(i["status"] == 0 for i in info), info
         got.append((H.effective(0), [H.field(0, k) for k in range(2)]))
@@ -41,6 +39,19 @@ def test_fp32_cg_matches_fp64_cg(grid, pass_mode):
     assert np.linalg.norm(c32 - c64) <= BOUND * np.linalg.norm(c64)
     for a, b in zip(e32, e64):
         assert np.linalg.norm(a - b) <= BOUND * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("pass_mode", [0, 2])
+@pytest.mark.parametrize("grid", GRIDS, ids=["x".join(map(str, g)) for g in GRIDS])
+def test_fp32_cg_matches_fp64_cg(grid, pass_mode):
+    from paper_1712_05145_gb300 import hom
+    _compare(grid, pass_mode, hom.HOM_CG)
+
+
+@pytest.mark.parametrize("n3", [1] + LENGTHS)
+def test_fp32_bicgstab_matches_fp64_cg(n3):
+    from paper_1712_05145_gb300 import hom
+    _compare((8, 6, n3), 0, hom.HOM_BICGSTAB)
 
 
 @pytest.mark.parametrize("grid", [(32, 24, 16), (128, 96, 128)])
