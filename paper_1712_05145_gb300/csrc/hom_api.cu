@@ -114,7 +114,7 @@ struct hom_ctx {
   bool zc_off[2] = {false, false};  // the autotuner found the single-CTA z pass faster
   bool zc_tma = false;         // FP32 cluster z pass: the TMA form (z_mode 0 and 2, or the autotuner's pick)
   bool y_tma = false;          // FP32 split y pass: the TMA form (y_mode 0 and 1, or the autotuner's pick)
-  unsigned* d_kerr = nullptr;  // bits set by kernels whose bounded waits gave up
+  unsigned* d_kerr = nullptr;  // bits set by kernels whose bounded waits gave up (in the slot before d_st)
   bool pc_off = false;         // the autotuner found the split x and y passes faster than the cluster ones
   bool tuned = false;
   void* d_bicg = nullptr;    // BiCGSTAB fields r_hat, v, s, t (the polarization scheme: eta)
@@ -227,23 +227,28 @@ size_t hat_bytes(const hom_ctx* c, int n) {
 hom_status ensure_cap(hom_ctx* c, int n) {
   if (n <= c->cap) return HOM_OK;
   const size_t ncta = ncta_max(c);
-  if (c->d_st) {
-    dfree(c, c->d_st, sizeof(RhsState) * c->cap);
+  if (c->cap) {
+    dfree(c, c->d_st - 1, sizeof(RhsState) * (c->cap + 1));
     dfree(c, c->d_part, sizeof(double) * 2 * c->cap * 2 * ncta);
     dfree(c, c->d_cnt, sizeof(unsigned) * 2 * c->cap);
     dfree(c, c->d_E, sizeof(double) * 6 * c->cap);
     dfree(c, c->d_mpart, sizeof(double) * (size_t)c->cap * 9 * c->mblk);
     dfree(c, c->d_mout, sizeof(double) * (size_t)c->cap * 9);
   }
-  c->cap = n;
-  CKS(dalloc(c, (void**)&c->d_st, sizeof(RhsState) * n));
+  c->cap = 0;   // until every array is there
+  c->d_kerr = nullptr;
+  // the slot in front of the states holds the kernels' error word: one copy reads both
+  CKS(dalloc(c, (void**)&c->d_st, sizeof(RhsState) * (n + 1)));
+  c->d_kerr = reinterpret_cast<unsigned*>(c->d_st);
+  c->d_st += 1;
   CKS(dalloc(c, (void**)&c->d_part, sizeof(double) * 2 * n * 2 * ncta));
   CKS(dalloc(c, (void**)&c->d_cnt, sizeof(unsigned) * 2 * n));
   CKS(dalloc(c, (void**)&c->d_E, sizeof(double) * 6 * n));
   CKS(dalloc(c, (void**)&c->d_mpart, sizeof(double) * (size_t)n * 9 * c->mblk));
   CKS(dalloc(c, (void**)&c->d_mout, sizeof(double) * (size_t)n * 9));
   CK(cudaMemsetAsync(c->d_cnt, 0, sizeof(unsigned) * 2 * n, c->stream));
-  CK(cudaMemsetAsync(c->d_st, 0, sizeof(RhsState) * n, c->stream));
+  CK(cudaMemsetAsync(c->d_st - 1, 0, sizeof(RhsState) * (n + 1), c->stream));
+  c->cap = n;
   return HOM_OK;
 }
 
@@ -490,22 +495,29 @@ hom_status ls_pass(hom_ctx* c, int nrhs, FwdArgs<Tf1, T> fa, ZArgs<T> za, InvArg
   return HOM_OK;
 }
 
-// Reads the kernels' error word (bits of bounded waits that gave up) and clears it.
+// Reports bits that kernels set when a bounded wait gave up (f: the error word just read), and clears them.
+hom_status kernel_flags(hom_ctx* c, unsigned f) {
+  if (f == 0) return HOM_OK;
+  CK(cudaMemsetAsync(c->d_kerr, 0, sizeof(unsigned), c->stream));
+  return fail(c, HOM_ERR_CUDA, "a kernel gave up a bounded wait (flags 0x%x): its results are invalid", f);
+}
 hom_status check_kernel_flags(hom_ctx* c) {
   if (!c->d_kerr) return HOM_OK;
   unsigned f = 0;
   CK(cudaMemcpyAsync(&f, c->d_kerr, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
-  if (f == 0) return HOM_OK;
-  CK(cudaMemsetAsync(c->d_kerr, 0, sizeof(unsigned), c->stream));
-  return fail(c, HOM_ERR_CUDA, "a kernel gave up a bounded wait (flags 0x%x): its results are invalid", f);
+  return kernel_flags(c, f);
 }
 
+// The first n loads' states, and the error word in front of them
 hom_status read_states(hom_ctx* c, int n, std::vector<RhsState>& h) {
-  h.resize(n);
-  CK(cudaMemcpyAsync(h.data(), c->d_st, sizeof(RhsState) * n, cudaMemcpyDeviceToHost, c->stream));
+  std::vector<RhsState> buf(n + 1);
+  CK(cudaMemcpyAsync(buf.data(), c->d_st - 1, sizeof(RhsState) * (n + 1), cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
-  return check_kernel_flags(c);
+  unsigned f;
+  std::memcpy(&f, buf.data(), sizeof f);
+  h.assign(buf.begin() + 1, buf.end());
+  return kernel_flags(c, f);
 }
 hom_status write_states(hom_ctx* c, const std::vector<RhsState>& h) {
   CK(cudaMemcpyAsync(c->d_st, h.data(), sizeof(RhsState) * h.size(), cudaMemcpyHostToDevice, c->stream));
@@ -2317,8 +2329,6 @@ HOM_API hom_status hom_create(const int32_t grid[3], const uint8_t* phase, int32
     if ((s = dalloc(c, (void**)&c->d_S64, b64 / 6 * c->S64_comps)) != HOM_OK) return bail(s);
   }
   if ((s = ensure_cap(c, 6)) != HOM_OK) return bail(s);
-  if ((s = dalloc(c, (void**)&c->d_kerr, sizeof(unsigned))) != HOM_OK) return bail(s);
-  if (cudaMemsetAsync(c->d_kerr, 0, sizeof(unsigned), c->stream) != cudaSuccess) return bail(HOM_ERR_CUDA);
   c->zc_tma = (c->opt.z_mode == 0 || c->opt.z_mode == 2);
   c->y_tma = (c->opt.y_mode != 2);
   if (cudaStreamSynchronize(c->stream) != cudaSuccess) return bail(HOM_ERR_CUDA);
