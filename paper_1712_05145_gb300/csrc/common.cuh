@@ -81,6 +81,21 @@ __device__ __forceinline__ df64 df_from_double(double d) {
   const float l = (float)lo * __uint_as_float((e - 948u) << 23);   // units of 2^(e - 1023 - 52)
   return df64(__uint_as_float(hi | s), s ? -l : l);
 }
+// A double rounded to the nearest float, and a float as a double, the same way (values out of the normal
+// FP32 range take the conversions)
+__device__ __forceinline__ float float_from_double(double d) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(d), a = u & 0x7fffffffffffffffull;
+  const unsigned e = (unsigned)(a >> 52);
+  if (e < 897u || e > 1150u) return (float)d;
+  const unsigned hi = (unsigned)((a + 0x0fffffffull + ((a >> 29) & 1ull)) >> 29) - (896u << 23);
+  return __uint_as_float(hi | ((unsigned)(u >> 32) & 0x80000000u));
+}
+__device__ __forceinline__ double to_double(float f) {
+  const unsigned u = __float_as_uint(f), e = (u >> 23) & 255u;
+  if (e == 0u || e == 255u) return (double)f;
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+}
+__device__ __forceinline__ double to_double(double d) { return d; }
 // a field value in the compute type T
 template <typename T> __device__ __forceinline__ T to_compute(double d) { return (T)d; }
 template <> __device__ __forceinline__ df64 to_compute<df64>(double d) { return df_from_double(d); }
