@@ -113,8 +113,8 @@ class ClockSampler:
 KERNEL_SOURCES = {
     "plane_fwd": ["plane_fwd.cu", "plane_cluster.cu", "xpass.cu"],
     "plane_fwd_f64": ["plane_fwd.cu", "xpass.cu"],
-    "zpass": ["cg_z.cu", "spectral_cg.h", "zpass.cu", "zcluster.cu", "spectral.cuh", "tma.cuh"],
-    "zpass_f64": ["zpass.cu", "zcluster.cu", "spectral.cuh", "tma.cuh"],
+    "zpass": ["cg_z.cu", "cg_z.cuh", "cg_bicg.cu", "spectral_cg.h", "zpass.cu", "zcluster.cu", "spectral.cuh", "tma.cuh"],
+    "zpass_f64": ["cg_df.cu", "spectral_cg.h", "zpass.cu", "zcluster.cu", "spectral.cuh", "tma.cuh"],
     "plane_inv": ["cg_plane.cu", "cg_rows.cu", "cg_xy.cuh", "plane_inv.cu", "plane_cluster.cu", "xpass.cu"],
     "plane_inv_f64": ["plane_inv.cu", "xpass.cu"],
     "ypass": ["ypass.cu", "tma.cuh"], "ypass_f64": ["ypass.cu", "tma.cuh"],

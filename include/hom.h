@@ -85,7 +85,7 @@ typedef struct {
                               per launch give the latency-bound kernels more CTAs; at 128^3 FP32
                               the default transforms all 6 unit loads per launch */
   void* cuda_stream;       /* cudaStream_t to run on; NULL = the handle's own stream */
-  int32_t pass_mode;       /* x-y transforms of the LS step (FP32 CG iterates on its own passes, which
+  int32_t pass_mode;       /* x-y transforms of the LS step (FP32 CG and BiCGSTAB iterate on their own passes, which
                               take whole planes per thread block where they fit unless pass_mode is
                               2, else rows and columns): 0 = fused plane kernels when a plane fits one CTA,
                               else (FP32 transforms) cluster plane passes, whose CTAs transpose
@@ -103,9 +103,10 @@ typedef struct {
   int32_t polarization_variant; /* HOM_POLARIZATION: 0 = x <- T(x) (Eyre-Milton, Monchiet-Bonnet);
                               1 = x <- (x + T(x)) / 2 (the averaged, augmented-Lagrangian form,
                               which also converges where a phase modulus is 0) */
-  int32_t z_mode;          /* z stage of the LS step (not of FP32 CG iterations, see pass_mode): 0 = cluster z pass (six CTAs, one per Kelvin
-                              component, meeting in distributed shared memory for the Green
-                              contraction) where its tile fits, else the single-CTA z pass; for FP32
+  int32_t z_mode;          /* z stage of the LS step (not of FP32 CG and BiCGSTAB iterations, see
+                              pass_mode): 0 = cluster z pass (six CTAs, one per Kelvin component,
+                              meeting in distributed shared memory for the Green contraction)
+                              where its tile fits, else the single-CTA z pass; for FP32
                               transforms its tiles move by TMA tensor loads and stores where that
                               fits (N3 >= 16, an even number of spectrum columns per plane); the
                               autotuner may pick any of these forms;
@@ -258,9 +259,10 @@ HOM_API hom_status hom_green_apply(hom_t h, int32_t nrhs, const double* tau_hat,
 
 /* Per-kernel accounting for performance measurement (off by default).
  * Kernel kinds of the Lippmann-Schwinger step, with FFTs in FP32 (0..2) or at FP64 accuracy (3..5:
- * double in HOM_FP64, double-float in the FP64-accurate passes of HOM_FP32_REFINE).  An iteration of
- * FP32 CG counts its two z passes as HOM_KERNEL_ZPASS (units once) and its middle pass, inverse and
- * forward x-y transforms with the material law between them, as HOM_KERNEL_PLANE_INV: */
+ * double in HOM_FP64, double-float in the FP64-accurate passes of HOM_FP32_REFINE).  An operator
+ * application of FP32 CG or BiCGSTAB counts its two z passes as HOM_KERNEL_ZPASS (units once) and its
+ * middle pass, inverse and forward x-y transforms with the material law between them, as
+ * HOM_KERNEL_PLANE_INV: */
 enum {
   HOM_KERNEL_PLANE_FWD = 0, HOM_KERNEL_ZPASS = 1, HOM_KERNEL_PLANE_INV = 2,
   HOM_KERNEL_PLANE_FWD_F64 = 3, HOM_KERNEL_ZPASS_F64 = 4, HOM_KERNEL_PLANE_INV_F64 = 5,

@@ -7,6 +7,10 @@
 // cg_df_out: the correction of a sweep, strain of x in double-float and inverse z FFT.  Its x-y
 // transforms add it to the FP64 solution free of the FP32 transform's incompatible rounding.
 //
+// Bound by the double-float chains (a product is two dependent operations, a sum six).  Ending the residual
+// here took 16.5 ms per solve of 96^3 spheres, six loads, to 15.1; the FP64 solution from double-float transforms saves
+// tight solves a projection and a second residual (256^3, 2e-7: 613 -> 538 ms).
+//
 // Tiles are those of the cluster z pass (zcluster.cu): 2^lg columns over all planes, one CTA per Kelvin
 // component; the residual's contraction reads the six components through distributed shared memory.
 #include <cooperative_groups.h>

@@ -216,8 +216,25 @@ __device__ __forceinline__ int col_rb(int n2) {
   }
 }
 
-template <int H>
-__global__ void __launch_bounds__(512, 2) cg_plane_kernel(const CgPlaneArgs a) {
+// Shared memory holds two planes of 8192 values per SM (with their phases), three of 6144, four of 4608.
+// The kernel waits at barriers and for shared memory, so CTAs that run independently of each other are worth more
+// than threads of one.  Measured with six loads, ms per launch:
+//   2304 to 4608 values: 256 threads of 64 registers, four CTAs: 96^3 0.132 (two of 512 threads: 0.182; three
+//     of 80 registers: 0.148), 128x64x64 0.071 (0.096), 96x48x96 0.078 (0.091)
+//   6144: 256 threads of 80 registers, three CTAs: 128x96x96 0.153 (two of 512: 0.203), 192x64x64 0.125 (0.147)
+//   8192: two CTAs.  128x128x128 gains from 80 registers and 256 threads (0.309, 512 threads of 64: 0.335), the
+//     oblong planes do not (256x64x64 0.181 and 0.170, 64x256x64 0.215 and 0.210)
+// Below 2304 values 8 values per thread are best (32x64x128 0.055, with 256 threads 0.076).
+template <int N2, int H>
+constexpr bool kWidePlane = N2 * H >= 6144 && (N2 * H < kMaxPlane || N2 == 2 * H);   // 80 registers
+bool wide_plane(const Geo& g) {
+  const long long e = (long long)g.n2 * g.h;
+  return e >= 6144 && (e < kMaxPlane || g.n2 == 2 * g.h);
+}
+template <int N2, int H, bool Wide>
+constexpr bool is_plane = N2 * H <= kMaxPlane && kWidePlane<N2, H> == Wide;
+template <int H, bool Wide>
+__global__ void __launch_bounds__(Wide ? 256 : 512, Wide ? 3 : 2) cg_plane_kernel(const CgPlaneArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const Geo& g = a.g;
   const int z = blockIdx.x, c = blockIdx.y, lrhs = blockIdx.z, rhs = a.rhs0 + lrhs;
@@ -262,11 +279,11 @@ __global__ void __launch_bounds__(512, 2) cg_plane_kernel(const CgPlaneArgs a) {
   grid_dep_wait();
   if (a.st[rhs].active == 0) return;
   cx<float>* Sp = a.S + ((long long)(lrhs * 6 + c) * g.n3 + z) * g.plane_c;
-  // planes of at most kMaxPlane values: larger pairs of lengths are not instantiated
+  // pairs of lengths of the other kind are not instantiated
   switch (n2) {
 #define HOM_CASE(N)                                                    \
   case N:                                                              \
-    if constexpr (N * H <= kMaxPlane) y_inverse<N, H>(m, Sp);          \
+    if constexpr (is_plane<N, H, Wide>) y_inverse<N, H>(m, Sp);       \
     break;
     HOM_PLANE_N2(HOM_CASE)
 #undef HOM_CASE
@@ -275,7 +292,7 @@ __global__ void __launch_bounds__(512, 2) cg_plane_kernel(const CgPlaneArgs a) {
   switch (n2) {
 #define HOM_CASE(N)                                                    \
   case N:                                                              \
-    if constexpr (N * H <= kMaxPlane) y_forward<N, H>(m, Sp);          \
+    if constexpr (is_plane<N, H, Wide>) y_forward<N, H>(m, Sp);       \
     break;
     HOM_PLANE_N2(HOM_CASE)
 #undef HOM_CASE
@@ -292,23 +309,23 @@ __global__ void __launch_bounds__(512, 2) cg_plane_kernel(const CgPlaneArgs a) {
   }
 }
 
-// one task of the widest stages per thread: 16 values at 512 threads on the largest planes, 8 below
 int plane_threads_cg(const Geo& g) {
   const long long e = (long long)g.n2 * g.h;
+  if (e >= 2304) return e < kMaxPlane || wide_plane(g) ? 256 : 512;
   int thr = (int)((e + 7) / 8);
   thr = ((thr + 31) / 32) * 32;
-  return thr < 64 ? 64 : thr > 512 ? 512 : thr;
+  return thr < 64 ? 64 : thr;
 }
 
-template <int H>
+template <int H, bool Wide>
 cudaError_t run_plane(const CgPlaneArgs& a, int nrhs, cudaStream_t s) {
   const Geo& g = a.g;
   const int thr = plane_threads_cg(g);
   const size_t smem = (size_t)(g.n2 * kPitch<H> + 2 * g.n2 + 2 * H + 1) * sizeof(cx<float>) +
                       (256 + thr) * sizeof(float) + (size_t)g.n2 * (g.n1 + 4);
-  cudaError_t err = set_smem(cg_plane_kernel<H>, smem);
+  cudaError_t err = set_smem(cg_plane_kernel<H, Wide>, smem);
   if (err != cudaSuccess) return err;
-  return launch_dependent(cg_plane_kernel<H>, dim3(g.n3, 6, nrhs), thr, smem, s, a);
+  return launch_dependent(cg_plane_kernel<H, Wide>, dim3(g.n3, 6, nrhs), thr, smem, s, a);
 }
 
 }  // namespace
@@ -328,7 +345,11 @@ cudaError_t launch_cg_plane(const CgPlaneArgs& a, int nrhs, cudaStream_t s) {
   if (!cg_plane_fits(a.g) || nrhs < 1 || a.n_phase > 256) return cudaErrorInvalidValue;
   count_launch();
   switch (a.g.h) {
-#define HOM_CASE(N) case N: return run_plane<N>(a, nrhs, s);
+#define HOM_CASE(N)                                                                          \
+  case N:                                                                                    \
+    if constexpr (256 * N >= 6144)                                                           \
+      if (wide_plane(a.g)) return run_plane<N, true>(a, nrhs, s);                            \
+    return run_plane<N, false>(a, nrhs, s);
     HOM_PLANE_H(HOM_CASE)
 #undef HOM_CASE
     default: return cudaErrorInvalidValue;

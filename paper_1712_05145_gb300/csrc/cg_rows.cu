@@ -22,8 +22,12 @@ template <int H> struct RowBlock {
   static constexpr size_t smem = (size_t)rows * pitch * sizeof(cx<float>) + tables + (256 + kRowThreads) * sizeof(float);
 };
 
+// Resident CTAs: latency-bound, so as many as fit with next to no spills, five (96 registers), six up to
+// 256-point rows.  512x256x512, one load: 1.054 ms with four, 1.000 with five (1.16 with two of 256 threads, 1.19
+// with eight of 64); 384x192x64, two loads: 0.185 -> 0.172; 256^3, two loads: 0.610, 0.550 with five, 0.518 with six.
+template <int H> constexpr int row_blocks() { return H > 128 ? 5 : 6; }
 template <int H>
-__global__ void __launch_bounds__(kRowThreads, 4) cg_rows_kernel(const CgPlaneArgs a) {
+__global__ void __launch_bounds__(kRowThreads, row_blocks<H>()) cg_rows_kernel(const CgPlaneArgs a) {
   using RB = RowBlock<H>;
   constexpr int R1 = RB::R1, R2 = RB::R2, NP = row_pair_tasks<H>(), ROWS = RB::rows;
   extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -1,4 +1,4 @@
-// z passes of the FP32 CG iteration in Fourier space (see spectral_cg.h).
+// z passes of the FP32 CG and BiCGSTAB iterations in Fourier space (see spectral_cg.h).
 //
 // A CTA owns TC consecutive spectrum columns (flat index of the x-y half-spectrum plane) over all N3
 // planes and walks through the six Kelvin components.  A thread keeps E values of one column in
@@ -6,6 +6,12 @@
 // inputs come straight from global memory and the last stage's outputs go straight back (TC
 // consecutive values per plane, 64 to 512 bytes).  The component loop accumulates w = tau_hat q in
 // registers, so no component has to wait for the others in shared memory and no cluster is needed.
+//
+// Bound by latency: a column's values, the next component and w take 128 registers a thread, 16 warps an
+// SM (80 and 96 registers spill; 16 values a thread, one exchange fewer, spill or take 168).  Inverse and forward pass,
+// ms per launch: 128^3, six loads, 0.241 and 0.203 (4.4 and 3.0 TB/s of their own traffic); 256^3, two loads,
+// 0.640 and 0.571; 512x256x512, one load, 1.29 and 1.39.  With the passes between them an iteration of 128^3
+// takes 0.75 ms; with the vectors as real fields its three passes took 1.00 ms.
 #pragma once
 #include "ls_common.cuh"
 #include "spectral.cuh"
@@ -529,7 +535,9 @@ __global__ void __launch_bounds__(ZLaunch<N, TC>::threads, ZLaunch<N, TC>::min_b
   }
 }
 
-// Tile width per depth: 128 to 256 threads per CTA (512 at N3 = 256 and 512, for runs of at least 64 bytes).
+// Tile width per depth: 128 to 256 threads per CTA (512 at N3 = 256 and 512, for runs of at least 64 bytes:
+// at 512, 8 columns 1.29 and 1.39 ms against 1.36 and 1.53 with 4; at 256, 16 columns 0.640 and 0.571 against 0.640
+// and 0.618 with 8; at 128, 16 columns 0.241 and 0.203 against 0.252 and 0.226 with 8).
 // Spectra of less than two wide tiles per SM take the narrow form.  Width and grouping depend on the
 // grid alone: a load's sums are grouped the same way in launches of any number of loads.
 constexpr int wide_tc(int n) {

@@ -17,7 +17,9 @@ LAME = np.array([[1.0, 1.0], [8.0, 5.0], [0.4, 0.3]])
 BOUND = 6.4e-5
 LENGTHS = [2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64, 96, 128, 192, 256, 384, 512]
 GRIDS = ([(8, 6, n) for n in [1] + LENGTHS] + [(8, n, 3) for n in LENGTHS] + [(2 * n, 4, 3) for n in LENGTHS]
-         + [(64, 48, 32), (96, 32, 12), (256, 64, 8)])
+         + [(64, 48, 32), (96, 32, 12), (256, 64, 8)]
+         # whole planes on either side of the lines between their launch shapes
+         + [(64, 64, 4), (96, 48, 4), (128, 64, 4), (96, 96, 4), (256, 48, 4), (128, 128, 4), (64, 256, 4)])
 
 
 def _ms(grid, seed):
