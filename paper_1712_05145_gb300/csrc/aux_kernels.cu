@@ -135,12 +135,16 @@ static int grid_for(long long n, int threads) {
 }
 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+// two voxels per thread where that leaves two blocks for every SM (below, more threads hide more latency)
+static bool two_voxels(long long M, int nf, const void* in, const void* out) {
+  return M % 2 == 0 && M * nf >= 2LL * 152 * 512 && aligned16(in) && aligned16(out);
+}
 
 // the internal side (work buffers) is always aligned; the caller's side may be any double array
 template <typename Tf>
 cudaError_t launch_mandel_to_kelvin(const double* in, Tf* out, long long M, int nf, cudaStream_t s) {
   count_launch();
-  if (M % 2 == 0 && aligned16(in) && aligned16(out))
+  if (two_voxels(M, nf, in, out))
     mandel_to_kelvin_kernel<Tf, 2><<<dim3(grid_for(M / 2, 256), nf), 256, 0, s>>>(in, out, M);
   else
     mandel_to_kelvin_kernel<Tf, 1><<<dim3(grid_for(M, 256), nf), 256, 0, s>>>(in, out, M);
@@ -149,7 +153,7 @@ cudaError_t launch_mandel_to_kelvin(const double* in, Tf* out, long long M, int 
 template <typename Tf>
 cudaError_t launch_kelvin_to_mandel(const Tf* in, double* out, long long M, int nf, cudaStream_t s) {
   count_launch();
-  if (M % 2 == 0 && aligned16(in) && aligned16(out))
+  if (two_voxels(M, nf, in, out))
     kelvin_to_mandel_kernel<Tf, 2><<<dim3(grid_for(M / 2, 256), nf), 256, 0, s>>>(in, out, M);
   else
     kelvin_to_mandel_kernel<Tf, 1><<<dim3(grid_for(M, 256), nf), 256, 0, s>>>(in, out, M);

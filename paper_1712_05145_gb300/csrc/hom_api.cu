@@ -465,7 +465,7 @@ hom_status ls_pass(hom_ctx* c, int nrhs, FwdArgs<Tf1, T> fa, ZArgs<T> za, InvArg
     ZArgs<T> zc = za;
     const int zi = sizeof(T) == 8 ? 1 : 0;
     if (za.mode == Z_GAMMA && za.ncomp_in == 6 && za.ncomp_out == 6 && c->opt.z_mode != 1 && !c->zc_off[zi] &&
-        zcluster_tiling<T>(zc, c->zc_lg[zi])) {
+        zcluster_tiling<T>(zc, c->zc_lg[zi], n)) {
       // one pass: six CTAs per tile, the contraction in distributed shared memory
       bool tma = false;
       if constexpr (std::is_same<T, float>::value) tma = c->zc_tma && ztma_fits(c->g, zc.tc_log2);

@@ -289,9 +289,9 @@ size_t zpass_smem_bytes(const Geo& g, size_t elem, int ncomp, int tc_log2) {
   return ((size_t)ncomp * cstride + g.n3) * elem;
 }
 
-// z-pass tile: 2^lg consecutive spectrum columns (lg <= 4; up to 8 on grids shallower than 16 planes, where 16
-// columns are too little work for a CTA: a two-dimensional cell's contraction kept 16 of 128 threads busy,
-// 0.22 ms at 512^2 in FP64, two loads) whose pencils fit kEPT elements per
+// z-pass tile: 2^lg consecutive spectrum columns (lg <= 4; up to 8 on two-dimensional cells whose tiles still
+// are two per SM, where 16 columns kept 16 of 128 threads of the contraction busy: 512^2 in FP64, two
+// loads, 0.220 -> 0.067 ms) whose pencils fit kEPT elements per
 // thread at <= 512 threads and <= 64 KB of shared memory.  Among the tiles whose row reads cover
 // at least one 32-byte sector, the one with the most resident warps per SM wins (ties: the
 // wider tile); at 128^3 in FP32 that is 4 columns (192 threads, 5 CTAs per SM) rather than 8
@@ -304,7 +304,8 @@ static int zpass_threads(int ncomp, int n3, int lg) {
 }
 
 bool zpass_tile_fits(const Geo& g, size_t elem, int ncomp, int lg) {
-  return lg >= 0 && lg <= (g.n3 < 16 ? 8 : 4) && (size_t)ncomp * g.n3 * ((size_t)1 << lg) <= (size_t)kEPT * 512 &&
+  return lg >= 0 && lg <= (g.n3 == 1 ? 8 : 4) && (lg <= 4 || g.plane_c >> lg >= 2 * 152) &&
+         (size_t)ncomp * g.n3 * ((size_t)1 << lg) <= (size_t)kEPT * 512 &&
          zpass_smem_bytes(g, elem, ncomp, lg) <= 64 * 1024;
 }
 

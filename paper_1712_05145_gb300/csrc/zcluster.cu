@@ -208,11 +208,12 @@ bool zcluster_tile_fits(const Geo& g, size_t elem, int lg) {
 }
 
 // Default width: grow the tile while it stays within about 256 threads, or while its runs along
-// the flat index are shorter than 128 bytes (one full memory transaction per z-plane); then, on
-// spectra of fewer tiles than the SMs hold, narrow it down to 64-byte runs (32^3 in FP64, one load: 54
-// CTAs of 64 columns on 152 SMs took 37 us, bound by the FP64 pipe of those SMs).
+// the flat index are shorter than 128 bytes (one full memory transaction per z-plane); then, where the
+// launch's nrhs loads have fewer CTAs than the SMs hold, narrow it to no less than 64-byte runs and 256 values
+// (32^3 in FP64, one load: 54 CTAs of 64 columns on 152 SMs took 37 us, bound by the FP64 pipe of those
+// SMs, 408 of 8 columns take 22; six loads fill the SMs with the wide tiles).
 template <typename T>
-bool zcluster_tiling(ZArgs<T>& a, int force_lg) {
+bool zcluster_tiling(ZArgs<T>& a, int force_lg, int nrhs) {
   const size_t elem = sizeof(cx<T>);
   if (a.g.n3 < 16) return false;   // shallow grids: the single-CTA z pass has more work per CTA
   int best = -1;
@@ -226,8 +227,8 @@ bool zcluster_tiling(ZArgs<T>& a, int force_lg) {
   }
   if (best < 0) return false;
   if (force_lg < 0)
-    while (best > 0 && ((size_t)1 << (best - 1)) * elem >= 64 &&
-           (a.g.plane_c + (1LL << best) - 1) / (1LL << best) * kZcComps < 2 * 152)
+    while (best > 0 && ((size_t)1 << (best - 1)) * elem >= 64 && (long long)a.g.n3 << (best - 1) >= 256 &&
+           (a.g.plane_c + (1LL << best) - 1) / (1LL << best) * kZcComps * nrhs < 2 * 152)
       --best;
   a.tc_log2 = best;
   const long long tc = 1LL << best;
@@ -239,9 +240,9 @@ bool zcluster_tiling(ZArgs<T>& a, int force_lg) {
   a.fd_in = make_fastdiv((unsigned)tc);
   return true;
 }
-template bool zcluster_tiling<float>(ZArgs<float>&, int);
-template bool zcluster_tiling<double>(ZArgs<double>&, int);
-template bool zcluster_tiling<df64>(ZArgs<df64>&, int);
+template bool zcluster_tiling<float>(ZArgs<float>&, int, int);
+template bool zcluster_tiling<double>(ZArgs<double>&, int, int);
+template bool zcluster_tiling<df64>(ZArgs<df64>&, int, int);
 
 template <typename T>
 cudaError_t launch_zcluster(const ZArgs<T>& a, int nrhs, cudaStream_t s) {

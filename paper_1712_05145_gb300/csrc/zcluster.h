@@ -11,7 +11,7 @@ namespace hom {
 // fd_in (division by the tile width).  force_lg >= 0 asks for tiles of 2^force_lg columns if
 // they fit.  Returns false when no tile fits (then the single-CTA z pass runs).
 template <typename T>
-bool zcluster_tiling(ZArgs<T>& a, int force_lg = -1);
+bool zcluster_tiling(ZArgs<T>& a, int force_lg = -1, int nrhs = 1);
 
 // Whether tiles of 2^lg columns fit the cluster z pass on this grid for element size elem.
 bool zcluster_tile_fits(const Geo& g, size_t elem, int lg);
