@@ -114,6 +114,17 @@ __global__ void __cluster_dims__(6, 1, 1) __launch_bounds__(kDfThreads, 1) cg_df
       a.r[o + 2 * cs] = mk<float>((float)v3.re, (float)v3.im);
     }
   }
+  if (tile == a.ntiles - 1) {
+    // The vector's last tile may hold columns past the plane.  The FP32 passes carry them along (with weight 0 in
+    // the sums, which a NaN would survive): zeros, whatever the buffer held before.
+    const int cols = (int)(((long long)a.vec_tiles << a.vec_lg) - g.plane_c);
+    for (int e = comp * nthr + tid; e < 3 * n3 * cols; e += 6 * nthr) {
+      const int rest = e / cols, i = rest / n3, n = rest - i * n3;
+      int cs;
+      const size_t o = vec_index(a, rhs, g.plane_c + (e - rest * cols), n, cs);
+      a.r[o + (size_t)i * cs] = mk<float>(0.0f, 0.0f);
+    }
+  }
   // |e|^2 = 2 |q|^2 |v|^2 + 2 |q . v|^2 and tr e = 2 q . v, as in cg_z_fwd
   red[tid] = (double)nn;
   red[nthr + tid] = (double)nd;
