@@ -16,6 +16,8 @@ cudaError_t launch_kelvin_to_mandel_inplace(double* f, long long M, int nf, cuda
 template <typename Tf>
 cudaError_t launch_cg_flush(Tf* x, const Tf* p, const RhsState* st, long long per, int n, cudaStream_t s);
 // x[i] += d[i] for i < n
+cudaError_t launch_scale(double* x, double s, long long n, cudaStream_t st);
+cudaError_t launch_max_abs(const double* x, long long n, double* out, cudaStream_t st);
 cudaError_t launch_add_correction(const float* d, double* x, long long n, cudaStream_t s);
 // x += a - b
 cudaError_t launch_add_difference(const float* a, const float* b, double* x, long long n, cudaStream_t s);

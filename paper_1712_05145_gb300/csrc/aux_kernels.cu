@@ -209,6 +209,39 @@ cudaError_t launch_add_difference(const float* a, const float* b, double* x, lon
   return cudaGetLastError();
 }
 
+// x *= s
+__global__ void scale_kernel(double* __restrict__ x, double s, long long n) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+    x[i] *= s;
+}
+cudaError_t launch_scale(double* x, double s, long long n, cudaStream_t st) {
+  count_launch();
+  scale_kernel<<<grid_for(n, 256), 256, 0, st>>>(x, s, n);
+  return cudaGetLastError();
+}
+
+// *out = max |x|, NaN where there is one: bit patterns of magnitudes are ordered as integers, NaN above all
+__global__ void max_abs_kernel(const double* __restrict__ x, long long n, unsigned long long* out) {
+  unsigned long long m = 0;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const unsigned long long a = (unsigned long long)__double_as_longlong(x[i]) & 0x7fffffffffffffffull;
+    if (a > m) m = a;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long a = __shfl_xor_sync(0xffffffffu, m, o);
+    if (a > m) m = a;
+  }
+  if ((threadIdx.x & 31) == 0) atomicMax(out, m);
+}
+cudaError_t launch_max_abs(const double* x, long long n, double* out, cudaStream_t st) {
+  cudaError_t e = cudaMemsetAsync(out, 0, sizeof(double), st);
+  if (e != cudaSuccess) return e;
+  count_launch();
+  max_abs_kernel<<<grid_for(n, 256), 256, 0, st>>>(x, n, reinterpret_cast<unsigned long long*>(out));
+  return cudaGetLastError();
+}
+
 // ---- spectrum layouts ------------------------------------------------------------
 // internal: per plane, n2 rows of h values (kx < n1/2) then the n2 Nyquist values;
 // standard: [n3][n2][n1/2 + 1] complex.  basis: 0 keep, 1 Mandel->Kelvin, 2 Kelvin->Mandel

@@ -1294,13 +1294,60 @@ hom_status literal_residual(hom_ctx* c, int n, const double* dE, const double* b
                  : literal_residual_t<Tf, double>(c, n, dE, b64, x64, r, act);
 }
 
-// Solves A x = b (Eq. cg_form) for n loads; b = -Gamma0 * (C : E) for Kelvin loads dE (order 0,
-// device [n][6]) or b = b64 (higher orders).  The solution x64 is FP64 in both precisions.
+// The FP32 sums of squares in Fourier space run over components |v|^2 ~ residual^2 / (2 M |q|^2), nine to fifteen
+// decades below the residual's square per voxel: with ||b|| = 1 they hold residuals down to 1e-13 at 512^3,
+// with ||b|| = 1e-12 none of a usual tolerance.  A x = b is linear, so a load whose ||b|| lies outside of
+// [2^-6, 2^20] is solved as 2^-k times itself, exactly, with ||b|| near 1: k from the norm, or from the load's
+// largest value where the norm under- or overflowed.  Marks in sel those of its loads that were scaled here (their
+// b is to be taken again), adds k to shift.  Order 0 (order0): the loads c->ord[0].loadsK, scaled in c->d_E; else b64.
+hom_status out_of_range_loads(hom_ctx* c, int n, bool order0, double* b64, const std::vector<RhsState>& st,
+                              std::vector<int>& shift, std::vector<int>& sel, bool& any) {
+  constexpr double kMin = 0x1p-12, kMax = 0x1p40;   // of ||b||^2
+  std::vector<double> E;
+  if (order0) {
+    E = c->ord[0].loadsK;
+    for (int i = 0; i < 6 * n; ++i) E[i] = std::ldexp(E[i], -shift[i / 6]);
+  }
+  any = false;
+  for (int i = 0; i < n; ++i) {
+    if (!sel[i]) continue;
+    sel[i] = 0;
+    const double b2 = st[i].b2;
+    if (b2 >= kMin && b2 <= kMax) continue;
+    int k = 0;
+    if (b2 > 0.0 && std::isfinite(b2)) {
+      k = (int)std::lround(0.5 * std::log2(b2));
+    } else {
+      double m = 0.0;
+      if (order0) {
+        for (int j = 0; j < 6; ++j) m = std::isnan(E[6 * i + j]) ? E[6 * i + j] : std::max(m, std::fabs(E[6 * i + j]));
+      } else {
+        CK(launch_max_abs(b64 + (size_t)i * 6 * c->g.M, 6 * c->g.M, c->d_mout, c->stream));
+        CK(cudaMemcpyAsync(&m, c->d_mout, sizeof m, cudaMemcpyDeviceToHost, c->stream));
+        CK(cudaStreamSynchronize(c->stream));
+      }
+      if (m > 0.0 && std::isfinite(m)) k = std::ilogb(m);   // else: a load of zeros, or one that ends as HOM_ERR_NUMERIC
+    }
+    k = std::max(-1000, std::min(1000, k));
+    if (k == 0) continue;
+    shift[i] += k;
+    sel[i] = 1;
+    any = true;
+    if (order0) for (int j = 0; j < 6; ++j) E[6 * i + j] = std::ldexp(E[6 * i + j], -k);
+    else CK(launch_scale(b64 + (size_t)i * 6 * c->g.M, std::ldexp(1.0, -k), 6 * c->g.M, c->stream));
+  }
+  if (any && order0) CK(cudaMemcpyAsync(c->d_E, E.data(), sizeof(double) * 6 * n, cudaMemcpyHostToDevice, c->stream));
+  return HOM_OK;
+}
+
+// Solves A x = b (Eq. cg_form) for n loads; b = -Gamma0 * (C : E) for the Kelvin loads dE = c->d_E of order 0
+// (device [n][6], also in c->ord[0].loadsK) or b = b64 (higher orders).  The solution x64 is FP64 in both
+// precisions; dE and b64 may be left scaled (out_of_range_loads).
 //  FP64 mode (Tf = double): Basic Scheme or CG in FP64 directly on x64.
 //  FP32 mode (Tf = float): iterative refinement -- each sweep runs FP32 CG on A d = r from d = 0
 //  (FP64 reductions), then x64 += d and an FP64 residual sweep restarts the next one.
 template <typename Tf>
-hom_status solve_system(hom_ctx* c, int n, const double* dE, const double* b64, double* x64, double tol,
+hom_status solve_system(hom_ctx* c, int n, const double* dE, double* b64, double* x64, double tol,
                         hom_solve_info* info) {
   const bool mixed = sizeof(Tf) == sizeof(float);
   CKS(ensure_cap(c, n));
@@ -1340,18 +1387,16 @@ hom_status solve_system(hom_ctx* c, int n, const double* dE, const double* b64, 
   // same verification in both precisions.
   const bool project = mixed || polar;
 
-  std::vector<RhsState> st(n);
-  for (int i = 0; i < n; ++i) {
-    RhsState s{};
-    s.tol = tol_inner;
-    s.max_iter = c->opt.max_iter;
-    s.active = 1;
-    s.restart = 1;
-    s.best = 1e300;
-    s.best_iter = 0;
-    s.stall = mixed ? 1 : 0;   // FP64 CG runs to the tolerance: a restart there only loses information
-    st[i] = s;
-  }
+  RhsState fresh{};
+  fresh.tol = tol_inner;
+  fresh.max_iter = c->opt.max_iter;
+  fresh.active = 1;
+  fresh.restart = 1;
+  fresh.best = 1e300;
+  fresh.best_iter = 0;
+  fresh.stall = mixed ? 1 : 0;   // FP64 CG runs to the tolerance: a restart there only loses information
+  std::vector<RhsState> st(n, fresh);
+  std::vector<int> shift(n, 0);   // load i is solved as 2^-shift[i] times itself
   CKS(write_states(c, st));
   std::vector<int> refine(n, 0), done(n, 0), act(n, 1);
 
@@ -1421,40 +1466,59 @@ hom_status solve_system(hom_ctx* c, int n, const double* dE, const double* b64, 
     CK(cudaMemsetAsync(x64, 0, tbytes<double>(c, n, 6), c->stream));
     if (mixed && !fourier) CK(cudaMemsetAsync(d, 0, fb, c->stream));
     // initial residual r = b (x = 0); FP32 CG takes it (and every restart's) in Fourier space
-    bool have_rh = false;   // the CG vector r holds the residual, not the real field
     CgDfArgs df;
     const bool df_z = fourier && cg_df_args(c, reinterpret_cast<cx<float>*>(vp), reinterpret_cast<cx<float>*>(vr),
                                             reinterpret_cast<cx<float>*>(vd), df);
-    if (fourier && dE != nullptr) {
-      CgPass q = cg_pass(c, reinterpret_cast<cx<float>*>(vp), nullptr, nullptr);
-      auto fa = fwd_args<float, float>(c, FWD_TAU, 6, 6);
-      fa.E = dE;
-      fa.st = c->d_st;
-      fa.S = q.za.S;
-      for (int r0 = 0; r0 < n; r0 += c->chunk) {
-        const int m = std::min(c->chunk, n - r0);
-        fa.rhs0 = q.za.rhs0 = r0;
-        CKS((fwd_xy<float, float>(c, fa, m)));
-        CKS(timed_launch(c, HOM_KERNEL_ZPASS, [&] { return launch_cg_z_fwd(q.za, CGF_RHS, m, c->stream); }));
+    bool have_rh = fourier && (dE != nullptr || df_z);   // the CG vector r holds the residual, not the real field
+    auto initial_residual = [&](const std::vector<int>& sel) {
+      if (fourier && dE != nullptr) {
+        CgPass q = cg_pass(c, reinterpret_cast<cx<float>*>(vp), nullptr, nullptr);
+        auto fa = fwd_args<float, float>(c, FWD_TAU, 6, 6);
+        fa.E = dE;
+        fa.st = c->d_st;
+        fa.S = q.za.S;
+        for (int r0 = 0; r0 < n; r0 += c->chunk) {
+          const int m = std::min(c->chunk, n - r0);
+          if (!any_of(sel, r0, m)) continue;
+          fa.rhs0 = q.za.rhs0 = r0;
+          CKS((fwd_xy<float, float>(c, fa, m)));
+          CKS(timed_launch(c, HOM_KERNEL_ZPASS, [&] { return launch_cg_z_fwd(q.za, CGF_RHS, m, c->stream); }));
+        }
+        return HOM_OK;
       }
-      have_rh = true;
-    } else if (df_z) {
-      CKS(cg_residual_fourier(c, n, nullptr, b64, nullptr, df, FIN_RHS, act));
-      have_rh = true;
-    } else if (dE != nullptr) {
-      auto fa = fwd_args<Tf, Tf>(c, FWD_TAU, 6, 6);
-      fa.E = dE;
-      fa.st = c->d_st;
-      auto za = z_args<Tf>(c, Z_GAMMA, 6, 6);
-      za.st = c->d_st;
-      auto ia = inv_args<Tf, Tf>(c, INV_STORE, FIN_RHS, 6, 6, 6);
-      ia.out = r;
-      ia.st = c->d_st;
-      CKS((ls_pass<Tf, Tf, Tf>(c, n, fa, za, ia)));
-    } else {
-      CKS(residual_sweep<Tf>(c, n, nullptr, b64, x64, r, FIN_RHS, nullptr));
-    }
+      if (df_z) return cg_residual_fourier(c, n, nullptr, b64, nullptr, df, FIN_RHS, sel);
+      if (dE != nullptr) {
+        auto fa = fwd_args<Tf, Tf>(c, FWD_TAU, 6, 6);
+        fa.E = dE;
+        fa.st = c->d_st;
+        auto za = z_args<Tf>(c, Z_GAMMA, 6, 6);
+        za.st = c->d_st;
+        auto ia = inv_args<Tf, Tf>(c, INV_STORE, FIN_RHS, 6, 6, 6);
+        ia.out = r;
+        ia.st = c->d_st;
+        return ls_pass<Tf, Tf, Tf>(c, n, fa, za, ia, &sel);
+      }
+      return residual_sweep<Tf>(c, n, nullptr, b64, x64, r, FIN_RHS, &sel);
+    };
+    CKS(initial_residual(act));
     CKS(read_states(c, n, st));
+    if (fourier) {
+      // a load whose norm left the range of the FP32 sums is solved as 2^-k times itself
+      std::vector<int> sel(n, 1);
+      for (int attempt = 0; attempt < 2; ++attempt) {   // the first norm may be that of an underflowed sum
+        bool any = false;
+        CKS(out_of_range_loads(c, n, dE != nullptr, b64, st, shift, sel, any));
+        if (!any) break;
+        for (int i = 0; i < n; ++i) {
+          if (sel[i]) st[i] = fresh;
+          else st[i].active = 0;
+        }
+        CKS(write_states(c, st));
+        CKS(initial_residual(sel));
+        CKS(read_states(c, n, st));
+      }
+      for (int i = 0; i < n; ++i) st[i].active = st[i].status == 0;
+    }
     for (int i = 0; i < n; ++i) {
       if (st[i].b2 == 0.0) {  // b = 0: x = 0 is exact
         done[i] = 1;
@@ -1611,6 +1675,8 @@ hom_status solve_system(hom_ctx* c, int n, const double* dE, const double* b64, 
       CKS(write_states(c, st));
       if (!again) break;
     }
+    for (int i = 0; i < n; ++i)
+      if (shift[i] != 0) CK(launch_scale(x64 + (size_t)i * 6 * c->g.M, std::ldexp(1.0, shift[i]), 6 * c->g.M, c->stream));
   }
 
   hom_status worst = HOM_OK;
