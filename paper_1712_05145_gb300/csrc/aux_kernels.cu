@@ -12,10 +12,12 @@ namespace hom {
 // ---- Mandel <-> Kelvin on real fields [nf][6][M] ------------------------------------
 // V consecutive voxels of one field per thread (V = 2 where the caller's pointer is 16-byte aligned: M is
 // even, so every component then is), one field per blockIdx.y: 72 B per voxel and field with an FP32 side,
-// 96 B in FP64.  With an FP32 side the conversions and sums were bound by the FP64 pipe (14 and 15
-// instructions of 16 cycles per warp), so types change by integer arithmetic on the bits and the sums
-// into FP32 run in double-float; those into FP64 keep nine FP64 instructions.  An FP32 step of two
-// 256x192x128 fields: 2.026 -> 1.991 ms (two voxels per thread alone: 2.023).
+// 96 B in FP64.  With an FP32 side the conversions are bound by the FP64 pipe (16 cycles per warp
+// instruction), so types change by integer arithmetic on the bits.  Into FP32 the three sums are formed in
+// FP64, as the FP64 step's are (terms may cancel); only their products with a constant run in double-float,
+// 48 bits in front of the rounding to 24 (equal to the FP64 product's rounding on 1.8e6 random voxels), on one
+// range test per voxel.  Those into FP64 keep nine FP64 instructions.  Two 256x192x128 fields into FP32: 0.204 ms;
+// 0.336 with FP64 products and conversions, 0.350 with FP64 products and integer conversions.
 template <typename T, int V> struct alignas(V * sizeof(T)) Voxels {
   T v[V];
 };
@@ -31,19 +33,24 @@ __global__ void __launch_bounds__(256) mandel_to_kelvin_kernel(const double* __r
     for (int c = 0; c < 6; ++c) m[c] = *reinterpret_cast<const Voxels<double, V>*>(a + c * M + i);
 #pragma unroll
     for (int j = 0; j < V; ++j) {
+      const double m0 = m[0].v[j], m1 = m[1].v[j], m2 = m[2].v[j], s = m0 + m1;
+      const double k0 = s + m2, k1 = m0 - m1, k2 = s - 2.0 * m2;
       if constexpr (sizeof(Tf) == 4) {
-        const df64 m0 = df_from_double(m[0].v[j]), m1 = df_from_double(m[1].v[j]), m2 = df_from_double(m[2].v[j]);
-        const df64 s = m0 + m1;
-        k[0].v[j] = (float)((s + m2) * df64(R3));
-        k[1].v[j] = (float)((m0 - m1) * df64(R2));
-        k[2].v[j] = (float)((s - df64(2.0f * m2.hi, 2.0f * m2.lo)) * df64(R6));
+        if (df_splits(k0) && df_splits(k1) && df_splits(k2)) {
+          k[0].v[j] = (float)(df_split(k0) * df64(R3));
+          k[1].v[j] = (float)(df_split(k1) * df64(R2));
+          k[2].v[j] = (float)(df_split(k2) * df64(R6));
+        } else {
+          k[0].v[j] = (float)(k0 * R3);
+          k[1].v[j] = (float)(k1 * R2);
+          k[2].v[j] = (float)(k2 * R6);
+        }
 #pragma unroll
         for (int c = 3; c < 6; ++c) k[c].v[j] = float_from_double(m[c].v[j]);
       } else {
-        const double m0 = m[0].v[j], m1 = m[1].v[j], m2 = m[2].v[j];
-        k[0].v[j] = (m0 + m1 + m2) * R3;
-        k[1].v[j] = (m0 - m1) * R2;
-        k[2].v[j] = (m0 + m1 - 2.0 * m2) * R6;
+        k[0].v[j] = k0 * R3;
+        k[1].v[j] = k1 * R2;
+        k[2].v[j] = k2 * R6;
 #pragma unroll
         for (int c = 3; c < 6; ++c) k[c].v[j] = m[c].v[j];
       }
