@@ -51,13 +51,22 @@ __device__ __forceinline__ df64 operator*(df64 a, df64 b) {
   e = __fmaf_rn(a.lo, b.hi, e);
   return df_fast_two_sum(p, e);
 }
-// a / b from the FP32 reciprocal of b.hi: one Newton step in double-float, the quotient, and its remainder's
-// correction (no FP64: a warp instruction takes 16 cycles of that pipe, a division some 20 of them)
+// a / b by long division with the FP32 reciprocal of b.hi: a quotient of two floats, its remainder a - b q with
+// every product and sum carried exactly down to the last terms, and one correction rounded into the low
+// float.  The error is that of the format, 2^-49, as of an FP64 quotient rounded to it.  (No FP64: a warp
+// instruction takes 16 cycles of that pipe, a division some 20 of them.)
 __device__ __forceinline__ df64 operator/(df64 a, df64 b) {
-  const float r0 = 1.0f / b.hi;
-  const df64 r = df64(r0) + (df64(1.0f) - b * df64(r0)) * df64(r0);
-  const df64 q = a * r, rem = a - b * q;
-  return q + df64(rem.hi * r0);
+  const float r = 1.0f / b.hi;
+  const float q1 = a.hi * r, p1 = __fmul_rn(b.hi, q1);   // __fmul_rn: not fused into the subtraction
+  const float q2 = (((a.hi - p1) - __fmaf_rn(b.hi, q1, -p1)) + __fmaf_rn(-b.lo, q1, a.lo)) * r;
+  const df64 q = df_fast_two_sum(q1, q2);
+  const float p = __fmul_rn(b.hi, q.hi), pe = __fmaf_rn(b.hi, q.hi, -p);
+  const float u = __fmul_rn(b.hi, q.lo), ue = __fmaf_rn(b.hi, q.lo, -u);
+  const float v = __fmul_rn(b.lo, q.hi), ve = __fmaf_rn(b.lo, q.hi, -v);
+  const df64 s1 = df_two_sum(a.hi - p, a.lo), s2 = df_two_sum(s1.hi, -pe), s3 = df_two_sum(s2.hi, -u),
+             s4 = df_two_sum(s3.hi, -v);   // a.hi - p is exact: they agree to some 22 bits
+  const float rem = s4.hi + (((s1.lo + s2.lo) + (s3.lo + s4.lo)) - (ue + __fmaf_rn(b.lo, q.lo, ve)));
+  return df_fast_two_sum(q.hi, __fmaf_rn(rem, r, q.lo));
 }
 __device__ __forceinline__ df64& operator+=(df64& a, df64 b) { return a = a + b; }
 __device__ __forceinline__ df64& operator-=(df64& a, df64 b) { return a = a - b; }

@@ -1,0 +1,54 @@
+"""Double-float operations of the FP32 mode's FP64-accurate passes against exact rational arithmetic.
+
+Two floats hold a number to 2^-49 of its size: the low one lies below half an ulp of the high one, 2^-24, and is
+rounded to 24 bits.  An FP64 operation rounded to two floats adds its own 2^-53, and the operations here are to be as
+good."""
+import ctypes
+import os
+import subprocess
+from fractions import Fraction
+
+import numpy as np
+import pytest
+
+from paper_1712_05145_gb300 import build
+
+pytestmark = pytest.mark.gpu
+BOUND = Fraction(1, 2 ** 49) + Fraction(1, 2 ** 53)
+N = 20000
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    so = tmp_path_factory.mktemp("df") / "double_float_ops.so"
+    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "double_float_ops.cu")
+    r = subprocess.run([build.nvcc()] + build.ARCH + build.FLAGS + ["-shared", src, "-o", str(so)],
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    return ctypes.CDLL(str(so))
+
+
+def _df(x):
+    """float64 array -> [n][2] float32, high and low part"""
+    hi = x.astype(np.float32)
+    return np.ascontiguousarray(np.stack([hi, (x - hi).astype(np.float32)], axis=1))
+
+
+def _exact(df):
+    return [Fraction(float(h)) + Fraction(float(l)) for h, l in df]
+
+
+def _ptr(a):
+    return ctypes.c_void_p(a.ctypes.data)
+
+
+@pytest.mark.parametrize("exponents", [(0, 0), (-20, 30), (30, -20)])
+def test_division(lib, exponents):
+    """Operands over eight binades each, of both signs, the kernels' 1 / |xi|^2 among them."""
+    rng = np.random.default_rng(3)
+    a, b = (_df(rng.choice([-1.0, 1.0], N) * 2.0 ** rng.uniform(e, e + 8, N)) for e in exponents)
+    a[:N // 2] = [1.0, 0.0]
+    out = np.zeros_like(a)
+    assert lib.df_divide(_ptr(a), _ptr(b), _ptr(out), N) == 0
+    worst = max(abs(q / (x / y) - 1) for q, x, y in zip(_exact(out), _exact(a), _exact(b)))
+    assert worst <= BOUND, float(worst * 2 ** 49)
