@@ -1295,14 +1295,20 @@ hom_status literal_residual(hom_ctx* c, int n, const double* dE, const double* b
 }
 
 // The FP32 sums of squares in Fourier space run over components |v|^2 ~ residual^2 / (2 M |q|^2), nine to fifteen
-// decades below the residual's square per voxel: with ||b|| = 1 they hold residuals down to 1e-13 at 512^3,
-// with ||b|| = 1e-12 none of a usual tolerance.  A x = b is linear, so a load whose ||b|| lies outside of
-// [2^-6, 2^20] is solved as 2^-k times itself, exactly, with ||b|| near 1: k from the norm, or from the load's
-// largest value where the norm under- or overflowed.  Marks in sel those of its loads that were scaled here (their
-// b is to be taken again), adds k to shift.  Order 0 (order0): the loads c->ord[0].loadsK, scaled in c->d_E; else b64.
-hom_status out_of_range_loads(hom_ctx* c, int n, bool order0, double* b64, const std::vector<RhsState>& st,
+// decades below the residual's square per voxel: at 512^3 and ||b|| = 1 they hold residuals down to 1e-13, at
+// ||b|| = 1e-12 none of a usual tolerance.  A x = b is linear, so a load whose squares at a quarter of the tolerance
+// (the closest that a sweep aims) would have less than 17 bits above the smallest FP32 number is solved as
+// 2^-k times itself, exactly, with ||b|| near 1: k from the norm, or from the load's largest value where the norm
+// under- or overflowed.  (Scaling every load below 2^-6 took the 64^3 order-1 problem, whose unit loads have ||b||
+// below that, from 41.07 to 41.68 ms: the residual is formed twice.)  Marks in sel those of its loads that were
+// scaled here (their b is to be taken again), adds k to shift.  Order 0 (order0): the loads c->ord[0].loadsK,
+// scaled in c->d_E; else b64.
+hom_status out_of_range_loads(hom_ctx* c, int n, bool order0, double tol, double* b64, const std::vector<RhsState>& st,
                               std::vector<int>& shift, std::vector<int>& sel, bool& any) {
-  constexpr double kMin = 0x1p-12, kMax = 0x1p40;   // of ||b||^2
+  const Geo& g = c->g;
+  const double q2 = 0.25 * (g.xs1 * g.xs1 * g.n1 * g.n1 + g.xs2 * g.xs2 * g.n2 * g.n2 + g.xs3 * g.xs3 * g.n3 * g.n3);
+  const double squares = 0x1p-132 * 2.0 * (double)g.M * q2;   // of a residual at the lower end
+  const double kMin = std::min(0x1p-12, squares / (0.0625 * tol * tol)), kMax = 0x1p40;   // of ||b||^2
   std::vector<double> E;
   if (order0) {
     E = c->ord[0].loadsK;
@@ -1507,7 +1513,7 @@ hom_status solve_system(hom_ctx* c, int n, const double* dE, double* b64, double
       std::vector<int> sel(n, 1);
       for (int attempt = 0; attempt < 2; ++attempt) {   // the first norm may be that of an underflowed sum
         bool any = false;
-        CKS(out_of_range_loads(c, n, dE != nullptr, b64, st, shift, sel, any));
+        CKS(out_of_range_loads(c, n, dE != nullptr, tol, b64, st, shift, sel, any));
         if (!any) break;
         for (int i = 0; i < n; ++i) {
           if (sel[i]) st[i] = fresh;

@@ -27,6 +27,7 @@ def test_order_1_does_not_read_what_earlier_calls_left_in_the_buffers(grid, sche
         assert all(i["status"] == 0 for i in H.solve(0, 1e-6))
         if poison:
             eps = torch.full((64, 6) + tuple(reversed(grid)), float("nan"), dtype=torch.float64, device="cuda")
+            torch.cuda.synchronize()   # the handle has a stream of its own
             hom.hom_ls_apply(H.h, 64, eps, None, eps)
             assert torch.isnan(eps).all()
         info = H.solve(1, 1e-6)

@@ -45,6 +45,7 @@ def test_differences_of_close_components_keep_their_digits(precision, offsets):
     ref = np.stack([oracle_ls_step_mandel(pb, pure[i], np.zeros(6)) for i in range(2)])
     H = hom.Homogenization(ms, precision=precision)
     src, dst = _at(torch.from_numpy(eps).cuda(), offsets[0]), _at(torch.zeros(SHAPE, dtype=torch.float64), offsets[1])
+    torch.cuda.synchronize()   # the handle has a stream of its own
     hom.hom_ls_apply(H.h, 2, src, None, dst)
     H.close()
     assert rel_err(dst.cpu().numpy(), ref) < TOL[precision]
@@ -60,6 +61,7 @@ def test_sums_whose_terms_exceed_fp32_are_finite_where_the_result_is(offset):
     eps[:, 0], eps[:, 1], eps[:, 2] = 2.5e38, 1e38, -1.5e38
     H = hom.Homogenization(ms, precision=1)
     src, dst = _at(eps.cuda(), offset), torch.full(SHAPE, 7.0, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()   # the handle has a stream of its own
     hom.hom_ls_apply(H.h, 2, src, None, dst)
     H.close()
     assert not dst.any()
@@ -75,6 +77,7 @@ def test_two_voxels_per_thread_match_the_oracle(scale, offset):
     ref = np.stack([oracle_ls_step_mandel(pb, eps[i], np.zeros(6)) for i in range(2)])
     H = hom.Homogenization(ms, precision=1)
     src, dst = _at(torch.from_numpy(scale * eps).cuda(), offset), _at(torch.zeros(SHAPE, dtype=torch.float64), offset)
+    torch.cuda.synchronize()   # the handle has a stream of its own
     hom.hom_ls_apply(H.h, 2, src, None, dst)
     H.close()
     assert rel_err(dst.cpu().numpy() / scale, ref) < TOL[1]
