@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
+
 #include "common.cuh"
 
 namespace hom {
@@ -27,7 +29,7 @@ struct Geo {
   int ty_log2, thr_y;    // y pass: 2^ty_log2 consecutive columns per CTA, threads
   FastDiv fd_ty;         // division by 2^ty_log2
   double xs1, xs2, xs3;  // physical frequency per integer wave number: 2 pi Nmax / N_i
-  df64 xsd[3];           // the same split in two floats
+  float xsw[3][3];       // the same as a sum of 15, 15 and 24 bits: wave numbers times the first two are exact in FP32
   // cluster plane passes (split grids, FP32 transforms): pc_Q CTAs per plane (0: not used), each
   // with pc_R = n2 / pc_Q rows and pc_Cb = h / pc_Q spectrum columns, pc_thr threads
   int pc_Q, pc_R, pc_Cb, pc_thr;
@@ -194,8 +196,23 @@ size_t plane_smem_bytes(const Geo& g, size_t elem);
 size_t zpass_smem_bytes(const Geo& g, size_t elem, int ncomp, int tc_log2);
 // fills fd_h, fd_n2 and the split-pass tiling of a geometry whose n1, n2, n3 are set
 void geo_finish(Geo& g);
-// the wave number scale of axes n1, n2, n3 (xs1 .. xsd)
-void geo_wave_scale(Geo& g);
+// the wave number scale of axes n1, n2, n3 (xs1 .. xsw)
+inline void geo_wave_scale(Geo& g) {
+  const int m = g.n2 > g.n3 ? g.n2 : g.n3, nmax = g.n1 > m ? g.n1 : m;
+  g.xs1 = 2.0 * M_PI * nmax / g.n1;
+  g.xs2 = 2.0 * M_PI * nmax / g.n2;
+  g.xs3 = 2.0 * M_PI * nmax / g.n3;
+  const double xs[3] = {g.xs1, g.xs2, g.xs3};
+  for (int i = 0; i < 3; ++i) {
+    int e;
+    std::frexp(xs[i], &e);
+    const double a = std::ldexp(std::floor(std::ldexp(xs[i], 15 - e)), e - 15);
+    const double b = std::ldexp(std::floor(std::ldexp(xs[i] - a, 30 - e)), e - 30);
+    g.xsw[i][0] = (float)a;
+    g.xsw[i][1] = (float)b;
+    g.xsw[i][2] = (float)(xs[i] - a - b);
+  }
+}
 // y pass tiles of 2^lg columns (ty_log2, thr_y, fd_ty); whether such tiles fit the y pass
 void set_ytile(Geo& g, int lg);
 bool ytile_fits(const Geo& g, int lg);

@@ -1,6 +1,4 @@
 // Forward plane pass of the Lippmann-Schwinger step (see ls_common.cuh).
-#include <cmath>
-
 #include "ls_common.cuh"
 
 namespace hom {
@@ -254,16 +252,6 @@ void geo_finish(Geo& g) {
   int lg = 0;
   while (lg < 4 && (g.h % (2 << lg)) == 0 && (long long)g.n2 * (2 << lg) <= (long long)kEPT * 512) ++lg;
   set_ytile(g, lg);
-}
-
-void geo_wave_scale(Geo& g) {
-  const int m = g.n2 > g.n3 ? g.n2 : g.n3, nmax = g.n1 > m ? g.n1 : m;
-  g.xs1 = 2.0 * M_PI * nmax / g.n1;
-  g.xs2 = 2.0 * M_PI * nmax / g.n2;
-  g.xs3 = 2.0 * M_PI * nmax / g.n3;
-  g.xsd[0] = df64(g.xs1);
-  g.xsd[1] = df64(g.xs2);
-  g.xsd[2] = df64(g.xs3);
 }
 
 bool ytile_fits(const Geo& g, int lg) {

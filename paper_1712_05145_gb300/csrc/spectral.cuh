@@ -57,17 +57,19 @@ __device__ __forceinline__ void green_consts_shared(T* dst, const double* c0, in
   }
 }
 
-// physical frequency of the integer wave number k on axis i: k xs, rounded once; without the FP64 pipe in
-// FP32 and double-float (k is exact in FP32)
+// physical frequency of the integer wave number k on axis i: k xs, rounded to T as an FP64 product would be,
+// without the FP64 pipe in FP32 and double-float (|k| <= 256 has 9 bits: k times 15 bits is exact)
 template <typename T> __device__ __forceinline__ T wave_scaled(const Geo& g, int i, int k) {
   return (T)(k * (i == 0 ? g.xs1 : i == 1 ? g.xs2 : g.xs3));
 }
 template <> __device__ __forceinline__ float wave_scaled<float>(const Geo& g, int i, int k) {
   const float f = (float)k;
-  return fmaf(f, g.xsd[i].hi, f * g.xsd[i].lo);
+  return fmaf(f, g.xsw[i][0], fmaf(f, g.xsw[i][1], f * g.xsw[i][2]));
 }
 template <> __device__ __forceinline__ df64 wave_scaled<df64>(const Geo& g, int i, int k) {
-  return df64((float)k) * g.xsd[i];
+  const float f = (float)k;
+  const df64 s = df_fast_two_sum(__fmul_rn(f, g.xsw[i][0]), __fmul_rn(f, g.xsw[i][1]));
+  return df_fast_two_sum(s.hi, fmaf(f, g.xsw[i][2], s.lo));
 }
 
 // The vector at which Gamma0_hat is evaluated for the half-spectrum frequency (kx, ky, n):

@@ -1,5 +1,5 @@
 // Double-float operations on arrays, for test_gpu_double_float.py: host arrays in and out, one value per thread.
-#include "common.cuh"
+#include "spectral.cuh"
 
 namespace {
 
@@ -8,6 +8,11 @@ using namespace hom;
 __global__ void divide_kernel(const df64* a, const df64* b, df64* out, int n) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] = a[i] / b[i];
+}
+
+__global__ void wave_kernel(const Geo g, int axis, int k0, int n, df64* out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) out[i] = wave_scaled<df64>(g, axis, k0 + i);
 }
 
 }  // namespace
@@ -20,6 +25,22 @@ extern "C" __attribute__((visibility("default"))) int df_divide(const df64* a, c
   cudaMemcpy(d + n, b, bytes, cudaMemcpyHostToDevice);
   divide_kernel<<<(n + 255) / 256, 256>>>(d, d + n, d + 2 * n, n);
   const cudaError_t e = cudaMemcpy(out, d + 2 * n, bytes, cudaMemcpyDeviceToHost);
+  cudaFree(d);
+  return e != cudaSuccess;
+}
+
+// wave numbers k0 .. k0 + n - 1 of an axis of the grid; *scale: the axis' frequency per wave number in FP64
+extern "C" __attribute__((visibility("default"))) int df_waves(const int* grid, int axis, int k0, int n, df64* out, double* scale) {
+  Geo g{};
+  g.n1 = grid[0];
+  g.n2 = grid[1];
+  g.n3 = grid[2];
+  geo_wave_scale(g);
+  *scale = axis == 0 ? g.xs1 : axis == 1 ? g.xs2 : g.xs3;
+  df64* d = nullptr;
+  if (cudaMalloc(&d, sizeof(df64) * n) != cudaSuccess) return 1;
+  wave_kernel<<<(n + 255) / 256, 256>>>(g, axis, k0, n, d);
+  const cudaError_t e = cudaMemcpy(out, d, sizeof(df64) * n, cudaMemcpyDeviceToHost);
   cudaFree(d);
   return e != cudaSuccess;
 }

@@ -52,3 +52,14 @@ def test_division(lib, exponents):
     assert lib.df_divide(_ptr(a), _ptr(b), _ptr(out), N) == 0
     worst = max(abs(q / (x / y) - 1) for q, x, y in zip(_exact(out), _exact(a), _exact(b)))
     assert worst <= BOUND, float(worst * 2 ** 49)
+
+
+@pytest.mark.parametrize("grid", [(512, 384, 96), (48, 512, 192), (12, 24, 512)])
+def test_wave_numbers(lib, grid):
+    g = (ctypes.c_int * 3)(*grid)
+    for axis in range(3):
+        n = 513
+        out, scale = np.zeros((n, 2), np.float32), ctypes.c_double()
+        assert lib.df_waves(g, axis, -256, n, _ptr(out), ctypes.byref(scale)) == 0
+        for k, x in zip(range(-256, 257), _exact(out)):
+            assert abs(x - k * Fraction(scale.value)) <= BOUND * abs(k) * Fraction(scale.value), (axis, k)
