@@ -91,7 +91,7 @@ __global__ void __cluster_dims__(6, 1, 1) __launch_bounds__(kDfThreads, 1) cg_df
       int kx, ky;
       freq_of(g, f, kx, ky);
       df64 x1, x2, x3;
-      wave_vector<df64>(g, a.green, a.gtab, kx, ky, n, x1, x2, x3);
+      cg_wave_vector<df64>(g, a.green, a.gtab, kx, ky, n, x1, x2, x3);
       kelvin_to_tensor<df64>(k, tt);
       tensor_dot_xi<df64>(tt, x1, x2, x3, w1, w2, w3);
       const df64 q = x1 * x1 + x2 * x2 + x3 * x3;
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(kDfThreads, 1) cg_df_out_kernel(const CgDfArgs
       int kx, ky, cs;
       freq_of(g, f, kx, ky);
       df64 q1, q2, q3;
-      wave_vector<df64>(g, a.green, a.gtab, kx, ky, n, q1, q2, q3);
+      cg_wave_vector<df64>(g, a.green, a.gtab, kx, ky, n, q1, q2, q3);
       const size_t o = vec_index(a, rhs, f, n, cs);
       cx<df64> v[3];
 #pragma unroll

@@ -140,33 +140,20 @@ template <int N, int TC> struct ZLaunch {
   static constexpr int min_blocks = threads >= resident ? 1 : resident / threads;
 };
 
-// wave vector q = (a1 cz(n), a2 cz(n), a3 sz(n)): the column factors, and the table over n
+// wave vector q = (a1 cz(n), a2 cz(n), a3 sz(n)), see cg_column_factors: the column factors, and the table over n
 struct ColumnQ {
   float a1, a2, a3;
 };
 // (In FP32 throughout: a warp instruction takes 16 cycles of the SM's FP64 pipe, and these run in every thread.)
 __device__ __forceinline__ ColumnQ column_q(const CgZArgs& a, int kx, int ky) {
-  const Geo& g = a.g;
   ColumnQ q;
-  if (a.green == 0) {
-    q.a1 = wave_scaled<float>(g, 0, kx == g.h ? 0 : kx);
-    q.a2 = wave_scaled<float>(g, 1, wave(ky, g.n2));
-    q.a3 = 1.0f;
-  } else {
-    const double* t2 = a.gtab + 2 * (g.h + 1);
-    const float s1 = (float)__ldg(a.gtab + kx), c1 = (float)__ldg(a.gtab + g.h + 1 + kx);
-    const float s2 = (float)__ldg(t2 + ky), c2 = (float)__ldg(t2 + g.n2 + ky);
-    q.a1 = s1 * c2;
-    q.a2 = c1 * s2;
-    q.a3 = c1 * c2;
-  }
+  cg_column_factors<float>(a.g, a.green, a.gtab, kx, ky, q.a1, q.a2, q.a3);
   return q;
 }
 __device__ __forceinline__ cx<float> z_factors(const CgZArgs& a, int n) {   // (cz, sz)
-  const Geo& g = a.g;
-  if (a.green == 0) return mk<float>(1.0f, wave_scaled<float>(g, 2, wave(n, g.n3)));
-  const double* t3 = a.gtab + 2 * (g.h + 1) + 2 * g.n2;
-  return mk<float>((float)__ldg(t3 + g.n3 + n), (float)__ldg(t3 + n));
+  cx<float> z;
+  cg_z_factors<float>(a.g, a.green, a.gtab, n, z.re, z.im);
+  return z;
 }
 
 __device__ __forceinline__ cx<float> fma_cx(cx<float> a, float s, cx<float> c) {

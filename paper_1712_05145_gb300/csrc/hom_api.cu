@@ -121,7 +121,7 @@ struct hom_ctx {
   std::vector<double> kelvin;  // [n_phase][4] host copy of the material table: C - C0, C
   double* d_polar64 = nullptr; // [n_phase][4] polarization-scheme table (c0 w, w), built on first use
   float* d_polar32 = nullptr;
-  double* d_gtab = nullptr;    // rotated finite-difference Green operator: sin, cos of pi j / N per axis
+  double* d_gtab = nullptr;    // rotated finite-difference Green operator: sin, cos, tan of pi j / N per axis
   int n_rve = 1;               // RVE slots of one grid (hom_options.n_rve)
   int rve_loads = 0;           // n_rve > 1: loads per slot (6, the unit loads); 0 with one RVE
   double* d_c0 = nullptr;      // n_rve > 1: [slot][4] (lambda0, mu0, 3 lambda0 + 2 mu0, 2 mu0)
@@ -2370,8 +2370,8 @@ HOM_API hom_status hom_create(const int32_t grid[3], const uint8_t* phase, int32
   if ((s = dalloc(c, (void**)&c->d_tw_df, sizeof(cx<df64>) * tdf.size())) != HOM_OK) return bail(s);
   cudaMemcpy(c->d_tw_df, tdf.data(), sizeof(cx<df64>) * tdf.size(), cudaMemcpyHostToDevice);
 
-  // the rotated finite-difference operator's per-axis table: sin(pi j / N), cos(pi j / N) by DFT index
-  // (j <= N1/2 on the half-spectrum axis), cos exactly 0 at j = N/2
+  // the rotated finite-difference operator's per-axis tables: sin(pi j / N), cos(pi j / N) by DFT index
+  // (j <= N1/2 on the half-spectrum axis), cos exactly 0 at j = N/2; then tan(pi j / N) of the three axes
   if (c->opt.green_operator == HOM_GREEN_ROTATED) {
     std::vector<double> gt;
     auto axis = [&](int n, int count) {
@@ -2381,6 +2381,12 @@ HOM_API hom_status hom_create(const int32_t grid[3], const uint8_t* phase, int32
     axis(n1, g.h + 1);
     axis(n2, n2);
     axis(n3, n3);
+    auto tangents = [&](int n, int count) {   // 0 at j = N/2, where no use is made of it
+      for (int j = 0; j < count; ++j) gt.push_back(2 * j == n ? 0.0 : std::tan(M_PI * j / n));
+    };
+    tangents(n1, g.h + 1);
+    tangents(n2, n2);
+    tangents(n3, n3);
     if ((s = dalloc(c, (void**)&c->d_gtab, sizeof(double) * gt.size())) != HOM_OK) return bail(s);
     cudaMemcpy(c->d_gtab, gt.data(), sizeof(double) * gt.size(), cudaMemcpyHostToDevice);
   }

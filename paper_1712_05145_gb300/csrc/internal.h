@@ -124,7 +124,7 @@ struct ZArgs {
   const double* c0;      //   c0[rve][4] = (lambda0, mu0, 3 lambda0 + 2 mu0, 2 mu0) in place of lam0, mu0
   double scale;          // factor applied with the spectral operator (1/M after a forward FFT)
   int green;             // 0: spectral wave vector; 1: rotated finite-difference vector q (gtab)
-  const double* gtab;    // green == 1: sin, cos of pi j / N per axis (see wave_vector)
+  const double* gtab;    // green == 1: sin, cos, tan of pi j / N per axis (see wave_vector, cg_column_factors)
   unsigned long long* prof;
   const cx<T>* tw_n3;
   unsigned* err;         // nullable: bits set by kernels whose bounded waits gave up (1) or whose

@@ -97,6 +97,55 @@ __device__ __forceinline__ void wave_vector(const Geo& g, int green, const doubl
   }
 }
 
+// The vector q of CG's vectors in Fourier space (strain v (x) q + q (x) v), q = (a1 cz, a2 cz, a3 sz) with the factors
+// of a spectrum column and of a z index.  Gamma0_hat depends on the direction of q alone, so any multiple will
+// do, as long as every pass takes the same:
+//  green == 0: xi, (a1, a2, a3) = (xi1, xi2, 1), (cz, sz) = (1, xi3);
+//  green == 1: the rotated symbol over cos cos cos, the tangents tan(pi j / N), which follow sin and cos in gtab:
+//  (t1, t2, 1) and (1, t3).  At a Nyquist index, where the tangent is infinite, the symbol's limit: the axis itself
+//  if it is the only one there, else 0.
+// So every component is one number rounded once to T, with either operator (as products of three rounded sines and
+// cosines those of the rotated one were off by up to 2.5 ulp in FP32).
+template <typename T> __device__ __forceinline__ T cg_tangent(const double* t) { return to_compute<T>(__ldg(t)); }
+template <typename T>
+__device__ __forceinline__ void cg_column_factors(const Geo& g, int green, const double* gtab, int kx, int ky, T& a1, T& a2,
+                                                  T& a3) {
+  if (green == 0) {
+    a1 = wave_scaled<T>(g, 0, kx == g.h ? 0 : kx);
+    a2 = wave_scaled<T>(g, 1, wave(ky, g.n2));
+    a3 = (T)1;
+  } else {
+    const double* t = gtab + 2 * (g.h + 1 + g.n2 + g.n3);
+    const bool nx = kx == g.h, ny = 2 * ky == g.n2;
+    a1 = ny ? (T)0 : nx ? (T)1 : cg_tangent<T>(t + kx);
+    a2 = nx ? (T)0 : ny ? (T)1 : cg_tangent<T>(t + g.h + 1 + ky);
+    a3 = nx || ny ? (T)0 : (T)1;
+  }
+}
+template <typename T>
+__device__ __forceinline__ void cg_z_factors(const Geo& g, int green, const double* gtab, int n, T& cz, T& sz) {
+  if (green == 0) {
+    cz = (T)1;
+    sz = wave_scaled<T>(g, 2, wave(n, g.n3));
+  } else {
+    const bool nz = 2 * n == g.n3;
+    cz = nz ? (T)0 : (T)1;
+    sz = nz ? (T)1 : cg_tangent<T>(gtab + 2 * (g.h + 1 + g.n2 + g.n3) + g.h + 1 + g.n2 + n);
+  }
+}
+template <typename T>
+__device__ __forceinline__ void cg_wave_vector(const Geo& g, int green, const double* gtab, int kx, int ky, int n, T& q1,
+                                               T& q2, T& q3) {
+  T cz, sz;
+  cg_column_factors<T>(g, green, gtab, kx, ky, q1, q2, q3);
+  cg_z_factors<T>(g, green, gtab, n, cz, sz);
+  if (green != 0) {   // cz and q3 are 0 or 1
+    q1 = cz == (T)0 ? (T)0 : q1;
+    q2 = cz == (T)0 ? (T)0 : q2;
+  }
+  q3 = q3 == (T)0 ? (T)0 : sz;
+}
+
 // eta_hat = -Gamma0_hat(xi) : tau_hat in Kelvin components, given w = tau_hat xi.
 // Gamma0_hat : tau_hat = v (x) xi + xi (x) v with
 // v = w / (2 mu0 |xi|^2) - (lam0 + mu0) / (2 mu0 (lam0 + 2 mu0)) (xi . w) xi / |xi|^4,

@@ -1,4 +1,5 @@
-"""Double-float operations of the FP32 mode's FP64-accurate passes against exact rational arithmetic.
+"""Double-float operations of the FP32 mode's FP64-accurate passes against exact rational arithmetic, and the wave
+vectors of its solvers.
 
 Two floats hold a number to 2^-49 of its size: the low one lies below half an ulp of the high one, 2^-24, and is
 rounded to 24 bits.  An FP64 operation rounded to two floats adds its own 2^-53, and the operations here are to be as
@@ -63,3 +64,24 @@ def test_wave_numbers(lib, grid):
         assert lib.df_waves(g, axis, -256, n, _ptr(out), ctypes.byref(scale)) == 0
         for k, x in zip(range(-256, 257), _exact(out)):
             assert abs(x - k * Fraction(scale.value)) <= BOUND * abs(k) * Fraction(scale.value), (axis, k)
+
+
+@pytest.mark.parametrize("grid", [(64, 48, 32), (24, 3, 16), (8, 6, 1), (256, 4, 2)])
+def test_rotated_wave_vectors(lib, grid):
+    """The rotated symbol p = (s1 c2 c3, c1 s2 c3, c1 c2 s3), s and c at pi j / N, up to a factor: tangents, each
+    rounded once to FP32 (2^-24, and some 2^-52 of the FP64 table and of p here); where a cosine is 0, the axis of p."""
+    axes = [np.arange(n) for n in (grid[0] // 2 + 1, grid[1], grid[2])]
+    sin = [np.sin(np.pi * j / n) for j, n in zip(axes, grid)]
+    cos = [np.where(2 * j == n, 0.0, np.cos(np.pi * j / n)) for j, n in zip(axes, grid)]
+    tan = [np.where(2 * j == n, 0.0, np.tan(np.pi * j / n)) for j, n in zip(axes, grid)]
+    tab = np.concatenate([v for s, c in zip(sin, cos) for v in (s, c)] + tan)
+    shape = tuple(len(a) for a in reversed(axes))
+    q = np.zeros(shape + (3,), np.float32)
+    assert lib.rotated_vectors((ctypes.c_int * 3)(*grid), _ptr(tab), len(tab), _ptr(q)) == 0
+    s3, s2, s1 = np.meshgrid(*reversed(sin), indexing="ij")
+    c3, c2, c1 = np.meshgrid(*reversed(cos), indexing="ij")
+    p = np.stack([s1 * c2 * c3, c1 * s2 * c3, c1 * c2 * s3], axis=-1)
+    c = (c1 * c2 * c3)[..., None]
+    inner = c[..., 0] != 0
+    assert np.all(np.abs(q * c - p)[inner] <= (2.0 ** -24 + 2.0 ** -48) * np.abs(p)[inner])
+    assert np.array_equal(q[~inner], (p != 0)[~inner].astype(np.float32))
