@@ -132,13 +132,14 @@ __device__ __forceinline__ void y_forward(const PlaneSmem& m, cx<float>* Sp) {
   }
 }
 
-// the rows of the plane: inverse, material law, forward (times 1/2 times 2, see cg_xy.cuh); returns the sum
-// of c p^2 / 2.  Consecutive threads take consecutive rows: the odd row pitch keeps them in distinct banks.
+// the rows of the plane: inverse, material law, forward (times 1/2 times 2, see cg_xy.cuh); returns the sum of
+// c p^2 / 2, at most 32 terms in a row in FP32 before a butterfly's sum joins the thread's others.  Consecutive
+// threads take consecutive rows: the odd row pitch keeps them in distinct banks.
 template <int H>
 __device__ __forceinline__ float rows(const PlaneSmem& m, const Geo& g) {
   constexpr int R1 = RowPlan<H>::R1, R2 = RowPlan<H>::R2, NP = row_pair_tasks<H>(), P = kPitch<H>;
   const int n2 = g.n2;
-  float acc = 0.0f;
+  float sum = 0.0f;
   for (int t = threadIdx.x; t < NP * n2; t += blockDim.x) {
     const int jp = (int)g.fd_n2.div((unsigned)t), row = t - jp * n2;
     cx<float>* q = m.pl + row * P;
@@ -167,6 +168,7 @@ __device__ __forceinline__ float rows(const PlaneSmem& m, const Geo& g) {
 #pragma unroll
     for (int s = 0; s < R2; ++s) v[s] = q[s];
     SmallDFT<float, R2, +1>::run(v);
+    float acc = 0.0f;
 #pragma unroll
     for (int s = 0; s < R2; ++s) {
       const uchar2 f = *reinterpret_cast<const uchar2*>(ph + 2 * R1 * s);
@@ -174,6 +176,7 @@ __device__ __forceinline__ float rows(const PlaneSmem& m, const Geo& g) {
       acc = fmaf(tau.re, v[s].re, fmaf(tau.im, v[s].im, acc));
       v[s] = tau;
     }
+    sum += acc;
     SmallDFT<float, R2, -1>::run(v);
 #pragma unroll
     for (int s = 0; s < R2; ++s) {
@@ -200,7 +203,7 @@ __device__ __forceinline__ float rows(const PlaneSmem& m, const Geo& g) {
     }
   }
   __syncthreads();
-  return acc;
+  return sum;
 }
 
 #define HOM_PLANE_N2(X) X(2) X(3) X(4) X(6) X(8) X(12) X(16) X(24) X(32) X(48) X(64) X(96) X(128) X(192) X(256)

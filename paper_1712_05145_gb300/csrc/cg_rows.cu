@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(kRowThreads, row_blocks<H>()) cg_rows_kernel(c
     }
   }
   __syncthreads();
-  float acc = 0.0f;
+  cx<float> acc = mk<float>(0.0f, 0.0f);   // of even and odd voxels, at most 32 terms in a row each
   for (int t = tid; t < R1 * nr; t += kRowThreads) {
     const int row = t / R1, b = t % R1;
     cx<float>* q = pl + row * RB::pitch + b * (R2 + 1);
@@ -91,7 +91,8 @@ __global__ void __launch_bounds__(kRowThreads, row_blocks<H>()) cg_rows_kernel(c
     for (int s = 0; s < R2; ++s) {
       const uchar2 f = *reinterpret_cast<const uchar2*>(ph + 2 * R1 * s);
       const cx<float> tau = mk<float>(tab[f.x] * v[s].re, tab[f.y] * v[s].im);
-      acc = fmaf(tau.re, v[s].re, fmaf(tau.im, v[s].im, acc));
+      acc.re = fmaf(tau.re, v[s].re, acc.re);
+      acc.im = fmaf(tau.im, v[s].im, acc.im);
       v[s] = tau;
     }
     SmallDFT<float, R2, -1>::run(v);
@@ -101,7 +102,7 @@ __global__ void __launch_bounds__(kRowThreads, row_blocks<H>()) cg_rows_kernel(c
       q[s] = v[s];
     }
   }
-  red[tid] = acc;
+  red[tid] = acc.re + acc.im;
   __syncthreads();
   for (int t = tid; t < NP * nr; t += kRowThreads) {
     const int row = t / NP, jp = t % NP, jb = jp == 0 ? R2 / 2 : R2 - jp;
