@@ -717,6 +717,22 @@ hom_status cg_iterations(hom_ctx* c, CgPass& q, int r0, int m, int iters) {
   return HOM_OK;
 }
 
+// BiCGSTAB's further vectors of n loads; its middle pass takes no energy
+hom_status bicg_vectors(hom_ctx* c, int n, CgPass& q) {
+  const size_t hb = hat_bytes(c, n);
+  if (c->bicg_bytes < 4 * hb) {
+    if (c->d_bicg) dfree(c, c->d_bicg, c->bicg_bytes);
+    c->d_bicg = nullptr;
+    c->bicg_bytes = 0;
+    CKS(dalloc(c, &c->d_bicg, 4 * hb));
+    c->bicg_bytes = 4 * hb;
+  }
+  cx<float>** vec[4] = {&q.za.rh, &q.za.v, &q.za.s, &q.za.t};
+  for (int i = 0; i < 4; ++i) *vec[i] = reinterpret_cast<cx<float>*>(reinterpret_cast<char*>(c->d_bicg) + i * hb);
+  q.pa.fin = FIN_NONE;
+  return HOM_OK;
+}
+
 // The same for BiCGSTAB (cg_bicg.cu), two operator applications per iteration
 hom_status bicg_iterations(hom_ctx* c, CgPass& q, int r0, int m, int iters) {
   q.za.rhs0 = q.pa.rhs0 = r0;
@@ -810,17 +826,7 @@ hom_status cg_sweep_fourier(hom_ctx* c, int n, const float* r, cx<float>* rh, cx
   CgPass q = cg_pass(c, rh, ph, xh);
   const bool bicg = c->opt.scheme == HOM_BICGSTAB;
   if (bicg) {
-    const size_t hb = hat_bytes(c, n);
-    if (c->bicg_bytes < 4 * hb) {
-      if (c->d_bicg) dfree(c, c->d_bicg, c->bicg_bytes);
-      c->d_bicg = nullptr;
-      c->bicg_bytes = 0;
-      CKS(dalloc(c, &c->d_bicg, 4 * hb));
-      c->bicg_bytes = 4 * hb;
-    }
-    cx<float>** vec[4] = {&q.za.rh, &q.za.v, &q.za.s, &q.za.t};
-    for (int i = 0; i < 4; ++i) *vec[i] = reinterpret_cast<cx<float>*>(reinterpret_cast<char*>(c->d_bicg) + i * hb);
-    q.pa.fin = FIN_NONE;
+    CKS(bicg_vectors(c, n, q));
     // its inner products are L2; the first pass restarts from r_hat = r, p = r
     for (auto& s : st) {
       s.rho = s.b2 * s.res_true * s.res_true;
@@ -900,16 +906,17 @@ hom_status cg_sweep_fourier(hom_ctx* c, int n, const float* r, cx<float>* rh, cx
 // that fit (the single-CTA z pass with tiles of 2^0 .. 2^4 columns, the cluster z pass with tiles
 // of at least 32 bytes per z-plane) and, on planes above one CTA, the cluster plane passes against
 // the split x and y passes; then the split y pass's tile width.  It tunes the passes of the
-// iteration precision T; FP32 CG handles take their loads per launch from timed CG iterations.
+// iteration precision T; FP32 CG and BiCGSTAB iterate on their own passes (spectral_cg.h), so their loads per
+// launch, and the y pass of planes above one CTA, are taken from timed iterations.
 // Tuning cache (HOM_TUNE_CACHE): one line per tuned handle kind,
-//   key: n1 n2 n3 precision transform-bytes z_mode pass_mode n_rve green chunk-capacity y_mode
+//   key: n1 n2 n3 precision transform-bytes z_mode pass_mode n_rve green chunk-capacity y_mode scheme
 //   value: chunk zc_off zc_lg ztile_lg pc_off ty_log2 zc_tma y_tma
 // The last line with a matching key wins.  A shape read back is one the tuner itself produced for
 // the same grid and options, so it is valid for this handle.
 std::string tune_key(const hom_ctx* c, size_t tbytes) {
   char b[192];
-  std::snprintf(b, sizeof(b), "%d %d %d %d %zu %d %d %d %d %d %d", c->g.n1, c->g.n2, c->g.n3, c->opt.precision, tbytes,
-                c->opt.z_mode, c->opt.pass_mode, c->n_rve, c->opt.green_operator, c->chunk, c->opt.y_mode);
+  std::snprintf(b, sizeof(b), "%d %d %d %d %zu %d %d %d %d %d %d %d", c->g.n1, c->g.n2, c->g.n3, c->opt.precision, tbytes,
+                c->opt.z_mode, c->opt.pass_mode, c->n_rve, c->opt.green_operator, c->chunk, c->opt.y_mode, c->opt.scheme);
   return b;
 }
 
@@ -935,7 +942,7 @@ bool tune_cache_load(hom_ctx* c, const char* path, const std::string& key, int i
   c->zc_lg[idx] = v[2];
   c->ztile_lg[idx] = v[3];
   c->pc_off = v[4] != 0;
-  if (c->g.split) set_ytile(c->g, v[5]);
+  if (ytile_fits(c->g, v[5])) set_ytile(c->g, v[5]);
   if (idx == 0) {
     c->zc_tma = v[6] != 0;
     c->y_tma = v[7] != 0;
@@ -1046,10 +1053,20 @@ hom_status autotune(hom_ctx* c) {
     c->zc_lg[idx] = best_lg;
     c->ztile_lg[idx] = -1;
   }
+  // ms of two passes over all nt loads, after one to warm up
+  auto time_of = [&](auto&& pass, float& ms) {
+    CKS(pass(1));
+    CK(cudaEventRecord(e0, c->stream));
+    CKS(pass(2));
+    CK(cudaEventRecord(e1, c->stream));
+    CK(cudaEventSynchronize(e1));
+    CK(cudaEventElapsedTime(&ms, e0, e1));
+    return HOM_OK;
+  };
   // then, where the split y pass runs, its tile width (2^2 .. 2^4 columns) and, for FP32
   // transforms, its tile copies (per-element asynchronous copies or TMA; y_mode 1 keeps TMA) with
   // the rest fixed
-  if (c->g.split && (c->g.pc_Q == 0 || c->pc_off || !std::is_same<T, float>::value)) {
+  auto tune_ypass = [&](auto&& pass) {
     constexpr bool f32 = std::is_same<T, float>::value;
     const int lg0 = c->g.ty_log2;
     const bool tma0 = f32 && c->y_tma;
@@ -1064,14 +1081,8 @@ hom_status autotune(hom_ctx* c) {
       set_ytile(c->g, lg);
       if (tma && !ytma_fits(c->g)) continue;
       if (f32) c->y_tma = tma;
-      CKS(apply_A<T>(c, nt, reinterpret_cast<const T*>(vin), reinterpret_cast<T*>(vout), nullptr));
-      CK(cudaEventRecord(e0, c->stream));
-      for (int rep = 0; rep < 2; ++rep)
-        CKS(apply_A<T>(c, nt, reinterpret_cast<const T*>(vin), reinterpret_cast<T*>(vout), nullptr));
-      CK(cudaEventRecord(e1, c->stream));
-      CK(cudaEventSynchronize(e1));
       float ms = 0.0f;
-      CK(cudaEventElapsedTime(&ms, e0, e1));
+      CKS(time_of(pass, ms));
       if (ms < best) {
         best = ms;
         best_y = lg;
@@ -1080,9 +1091,18 @@ hom_status autotune(hom_ctx* c) {
     }
     set_ytile(c->g, best_y);
     if (f32) c->y_tma = best_tma;
-  }
-  // FP32 CG iterates on its own passes (spectral_cg.h): its loads per launch are timed on them
-  if (std::is_same<T, float>::value && c->opt.scheme == HOM_CG) {
+    return HOM_OK;
+  };
+  const bool bicg = c->opt.scheme == HOM_BICGSTAB;
+  const bool fourier = std::is_same<T, float>::value && (c->opt.scheme == HOM_CG || bicg);
+  if (!fourier) {
+    if (c->g.split && (c->g.pc_Q == 0 || c->pc_off || !std::is_same<T, float>::value))
+      CKS(tune_ypass([&](int reps) {
+        for (int i = 0; i < reps; ++i)
+          CKS(apply_A<T>(c, nt, reinterpret_cast<const T*>(vin), reinterpret_cast<T*>(vout), nullptr));
+        return HOM_OK;
+      }));
+  } else {
     void* vec[3];
     const int slot[3] = {0, 1, 3};
     const size_t hb = hat_bytes(c, nt);
@@ -1094,24 +1114,34 @@ hom_status autotune(hom_ctx* c) {
     CKS(write_states(c, st));
     CgPass q = cg_pass(c, reinterpret_cast<cx<float>*>(vec[0]), reinterpret_cast<cx<float>*>(vec[1]),
                        reinterpret_cast<cx<float>*>(vec[2]));
+    if (bicg) {
+      CKS(bicg_vectors(c, nt, q));
+      CK(cudaMemsetAsync(c->d_bicg, 0, c->bicg_bytes, c->stream));
+    }
+    auto sweep = [&](int iters) {
+      for (int r0 = 0; r0 < nt; r0 += c->chunk) {
+        const int m = std::min(c->chunk, nt - r0);
+        CKS(bicg ? bicg_iterations(c, q, r0, m, iters) : cg_iterations(c, q, r0, m, iters));
+      }
+      return HOM_OK;
+    };
+    if (!q.whole_planes) {
+      float ms = 0.0f;
+      CKS(time_of(sweep, ms));
+      best = ms;
+      CKS(tune_ypass(sweep));
+    }
     best = 1e300;
     for (int ck : chunks) {
-      auto sweep = [&](int iters) {
-        for (int r0 = 0; r0 < nt; r0 += ck) CKS(cg_iterations(c, q, r0, std::min(ck, nt - r0), iters));
-        return HOM_OK;
-      };
-      CKS(sweep(1));   // warm-up
-      CK(cudaEventRecord(e0, c->stream));
-      CKS(sweep(2));
-      CK(cudaEventRecord(e1, c->stream));
-      CK(cudaEventSynchronize(e1));
+      c->chunk = ck;
       float ms = 0.0f;
-      CK(cudaEventElapsedTime(&ms, e0, e1));
+      CKS(time_of(sweep, ms));
       if (ms < best) {
         best = ms;
-        c->chunk = ck;
+        best_chunk = ck;
       }
     }
+    c->chunk = best_chunk;
   }
   c->ev_pool.push_back(e0);
   c->ev_pool.push_back(e1);
