@@ -386,23 +386,26 @@ HOM_API void hom_server_destroy(hom_server_t s);
 /* Bytes of device memory the handle holds now. */
 HOM_API int64_t hom_device_bytes(hom_t h);
 
-/* Launch shape of the handle's iteration passes: loads transformed per launch and the z-pass
- * tile width as log2 of its columns (-1: chosen per launch by the occupancy rule).  After an
- * autotuned solve these are the tuned values.  Pointers nullable. */
+/* Launch shape of the handle's passes: loads transformed per launch and the z-pass tile width as
+ * log2 of its columns (-1: chosen per launch by the occupancy rule).  After an autotuned solve
+ * these are the tuned values.  The tile widths and forms here and below are those of the LS step
+ * (hom_ls_apply, the Basic and polarization schemes, FP64 solvers); FP32 CG and BiCGSTAB iterate on
+ * passes of their own (hom_options.pass_mode).  Pointers nullable. */
 HOM_API hom_status hom_launch_config(hom_t h, int32_t* loads_per_launch, int32_t* ztile_log2);
 
-/* x-y passes of the handle's FP32 transforms: *cluster_ctas = CTAs per plane of the cluster plane
+/* x-y passes of the LS step's FP32 transforms: *cluster_ctas = CTAs per plane of the cluster plane
  * passes (hom_options.pass_mode), 0 when the fused plane kernels or the split x and y passes run. */
 HOM_API hom_status hom_plane_config(hom_t h, int32_t* cluster_ctas);
 
-/* split y pass of the handle's iteration passes: *tile_log2 its tile width as log2 of its columns
+/* split y pass of the LS step: *tile_log2 its tile width as log2 of its columns
  * (-1 when the grid's x-y transforms are not split), *tma = 1 when its FP32 tiles move by TMA tensor
  * loads and stores (hom_options.y_mode and the autotuner's pick).  Pointers nullable. */
 HOM_API hom_status hom_ypass_config(hom_t h, int32_t* tile_log2, int32_t* tma);
 
-/* z stage of the handle's iteration passes: *cluster = 1 for the cluster z pass, 2 for its TMA
- * form, 0 for the single-CTA z pass (hom_options.z_mode); *tile_log2 its tile width as log2 of its
- * columns (-1: the default rule).  Pointers nullable. */
+/* z stage of the LS step: *cluster = 1 for the cluster z pass, 2 for its TMA form, 0 for the
+ * single-CTA z pass (hom_options.z_mode); *tile_log2 its tile width as log2 of its columns (-1: the
+ * default rule), which depends on the loads of a launch: those of the handle's last step, six
+ * before the first.  Pointers nullable. */
 HOM_API hom_status hom_zpass_config(hom_t h, int32_t* cluster, int32_t* tile_log2);
 
 /* Kernels this library has launched in this process so far, over all handles, servers and the

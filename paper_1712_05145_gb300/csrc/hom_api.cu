@@ -111,6 +111,7 @@ struct hom_ctx {
   void* d_work[4] = {nullptr, nullptr, nullptr, nullptr};
   int ztile_lg[2] = {-1, -1};  // z-pass tile width forced by the autotuner (FP32, FP64); -1: rule
   int zc_lg[2] = {-1, -1};     // cluster z-pass tile width forced by the autotuner; -1: rule
+  int z_loads[2] = {6, 6};     // loads of the last z pass (FP32, FP64), which the cluster form's tile width depends on
   bool zc_off[2] = {false, false};  // the autotuner found the single-CTA z pass faster
   bool zc_tma = false;         // FP32 cluster z pass: the TMA form (z_mode 0 and 2, or the autotuner's pick)
   bool y_tma = false;          // FP32 split y pass: the TMA form (y_mode 0 and 1, or the autotuner's pick)
@@ -464,6 +465,7 @@ hom_status ls_pass(hom_ctx* c, int nrhs, FwdArgs<Tf1, T> fa, ZArgs<T> za, InvArg
     CKS(fwd_xy<Tf1, T>(c, fa, n));
     ZArgs<T> zc = za;
     const int zi = sizeof(T) == 8 ? 1 : 0;
+    if (r0 == 0) c->z_loads[zi] = n;
     if (za.mode == Z_GAMMA && za.ncomp_in == 6 && za.ncomp_out == 6 && c->opt.z_mode != 1 && !c->zc_off[zi] &&
         zcluster_tiling<T>(zc, c->zc_lg[zi], n)) {
       // one pass: six CTAs per tile, the contraction in distributed shared memory
@@ -2134,7 +2136,8 @@ HOM_API hom_status hom_zpass_config(hom_t c, int32_t* cluster, int32_t* tile_log
   p32.g = c->g;
   p64.g = c->g;
   bool on = c->opt.z_mode != 1 && !c->zc_off[zi];
-  if (on) on = c->fp32 ? zcluster_tiling<float>(p32, c->zc_lg[zi]) : zcluster_tiling<double>(p64, c->zc_lg[zi]);
+  if (on) on = c->fp32 ? zcluster_tiling<float>(p32, c->zc_lg[zi], c->z_loads[zi])
+                       : zcluster_tiling<double>(p64, c->zc_lg[zi], c->z_loads[zi]);
   const bool tma = on && c->fp32 && c->zc_tma && ztma_fits(c->g, p32.tc_log2);
   if (cluster) *cluster = tma ? 2 : (on ? 1 : 0);
   if (tile_log2) *tile_log2 = on ? (c->fp32 ? p32.tc_log2 : p64.tc_log2) : c->ztile_lg[zi];

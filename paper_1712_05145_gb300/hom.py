@@ -397,7 +397,7 @@ def hom_device_bytes(h):
 
 
 def hom_launch_config(h):
-    """(loads per launch, z-pass tile log2 width or -1) of a handle's iteration passes."""
+    """(loads per launch, z-pass tile log2 width or -1) of a handle's passes."""
     a, b = ctypes.c_int32(), ctypes.c_int32()
     _check(h, load_library().hom_launch_config(h, ctypes.byref(a), ctypes.byref(b)))
     return a.value, b.value
@@ -420,15 +420,15 @@ def hom_plane_config(h):
 
 
 def hom_ypass_config(h):
-    """(tile log2 width or -1, 1 if its FP32 tiles move by TMA else 0) of a handle's split y pass."""
+    """(tile log2 width or -1, 1 if its FP32 tiles move by TMA else 0) of the LS step's split y pass."""
     a, b = ctypes.c_int32(), ctypes.c_int32()
     _check(h, load_library().hom_ypass_config(h, ctypes.byref(a), ctypes.byref(b)))
     return a.value, b.value
 
 
 def hom_zpass_config(h):
-    """(z stage, tile log2 width or -1) of a handle's iteration passes; the z stage is 1 for the
-    cluster z pass, 2 for its TMA form, 0 for the single-CTA z pass."""
+    """(z stage, tile log2 width or -1) of a handle's LS step with the loads of its last one (six before
+    the first); the z stage is 1 for the cluster z pass, 2 for its TMA form, 0 for the single-CTA z pass."""
     a, b = ctypes.c_int32(), ctypes.c_int32()
     _check(h, load_library().hom_zpass_config(h, ctypes.byref(a), ctypes.byref(b)))
     return a.value, b.value
