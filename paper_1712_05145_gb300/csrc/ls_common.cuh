@@ -45,6 +45,11 @@ template <> struct PlaneCfg<df64> {
 template <typename T> constexpr bool kRealCg = std::is_same<T, double>::value;
 // FP32 transforms whose epilogue adds to an FP64 field (INV_ADD): a kernel of its own
 template <typename Tf, typename T> constexpr bool kInvAdds = sizeof(Tf) == 8 && sizeof(T) == 4;
+// whether the kernels of these types have a mode (a launch of another one is refused)
+template <typename T> bool fwd_mode_ok(int mode) { return mode != FWD_CG || kRealCg<T>; }
+template <typename Tf, typename T> bool inv_mode_ok(int mode) {
+  return kInvAdds<Tf, T> ? mode == INV_ADD : mode == INV_STORE || (mode == INV_CG && kRealCg<T>);
+}
 // threads of a plane CTA: every element of the n2 x h plane has a slot, whole warps, >= 128
 template <typename T>
 inline int plane_threads(const Geo& g) {
@@ -114,10 +119,6 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
 }
 
-// Prefetch of the 128-byte line of an address into L2.
-__device__ __forceinline__ void prefetch_line_l2(const void* ptr) {
-  asm volatile("prefetch.global.L2 [%0];" ::"l"(ptr));
-}
 // Bulk prefetch of a contiguous global range into L2 (TMA, sm_90+).  bytes must be a multiple
 // of 16 and ptr 16-byte aligned; the range must lie inside one allocation.  Issued by one thread.
 __device__ __forceinline__ void prefetch_l2(const void* ptr, unsigned bytes) {

@@ -435,10 +435,11 @@ static cudaError_t launch_cluster(K kernel, const A& a, int nrhs, int ncomp, cud
 }
 
 cudaError_t launch_plane_fwd_cluster(const FwdArgs<float, float>& a, int nrhs, cudaStream_t s) {
-  if (a.n_phase > 256) return cudaErrorInvalidValue;
+  if (a.n_phase > 256 || !fwd_mode_ok<float>(a.mode)) return cudaErrorInvalidValue;
   return launch_cluster(plane_fwd_cluster_kernel<float, float, kEPT>, a, nrhs, a.ncomp, s);
 }
 cudaError_t launch_plane_inv_cluster(const InvArgs<float, float>& a, int nrhs, cudaStream_t s) {
+  if (!inv_mode_ok<float, float>(a.mode)) return cudaErrorInvalidValue;
   return launch_cluster(plane_inv_cluster_kernel<float, float, kEPT>, a, nrhs, a.ncomp, s);
 }
 

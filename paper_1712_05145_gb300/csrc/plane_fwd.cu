@@ -335,7 +335,7 @@ template <typename Tf, typename T>
 cudaError_t launch_plane_fwd(const FwdArgs<Tf, T>& a, int nrhs, cudaStream_t s) {
   const int thr = plane_threads<T>(a.g);
   if ((long long)a.g.n2 * a.g.h > (long long)PlaneCfg<T>::kEPT * thr || thr > PlaneCfg<T>::kMaxThreads ||
-      a.n_phase > 256)
+      a.n_phase > 256 || !fwd_mode_ok<T>(a.mode))
     return cudaErrorInvalidValue;
   const size_t smem = plane_smem_bytes(a.g, sizeof(cx<T>));
   auto k = plane_fwd_kernel<Tf, T, PlaneCfg<T>::kEPT>;

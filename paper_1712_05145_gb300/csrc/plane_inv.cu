@@ -190,7 +190,8 @@ plane_inv_kernel(const InvArgs<Tf, T> a) {
 template <typename Tf, typename T>
 cudaError_t launch_plane_inv(const InvArgs<Tf, T>& a, int nrhs, cudaStream_t s) {
   const int thr = plane_threads<T>(a.g);
-  if ((long long)a.g.n2 * a.g.h > (long long)PlaneCfg<T>::kEPT * thr || thr > PlaneCfg<T>::kMaxThreads)
+  if ((long long)a.g.n2 * a.g.h > (long long)PlaneCfg<T>::kEPT * thr || thr > PlaneCfg<T>::kMaxThreads ||
+      !inv_mode_ok<Tf, T>(a.mode))
     return cudaErrorInvalidValue;
   const size_t smem = plane_smem_bytes(a.g, sizeof(cx<T>));
   auto k = plane_inv_kernel<Tf, T, PlaneCfg<T>::kEPT>;

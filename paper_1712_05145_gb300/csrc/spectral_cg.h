@@ -28,7 +28,6 @@ struct CgZArgs {
   int rve_loads;
   const double* c0;        // several RVE slots: [rve][4], see ZArgs
   float scale;             // 1 / M, the factor of the forward transform
-  float xs[3];             // Geo's xs1, xs2, xs3
   int green;
   const double* gtab;
   const cx<float>* tw_n3;
@@ -103,6 +102,5 @@ bool cg_plane_fits(const Geo& g);
 cudaError_t launch_cg_plane(const CgPlaneArgs& a, int nrhs, cudaStream_t s);
 int cg_row_blocks(const Geo& g);          // CTAs of one (load, component) in cg_rows
 cudaError_t launch_cg_rows(const CgPlaneArgs& a, int nrhs, cudaStream_t s);
-
 
 }  // namespace hom

@@ -391,7 +391,8 @@ static size_t xpass_smem_bytes(const Geo& g, size_t elem) {
 
 template <typename Tf, typename T>
 cudaError_t launch_xpass_fwd(const FwdArgs<Tf, T>& a, int nrhs, cudaStream_t s) {
-  if ((long long)a.g.rb * a.g.h > (long long)kEPT * a.g.thr_x || a.g.thr_x > 256 || a.n_phase > 256)
+  if ((long long)a.g.rb * a.g.h > (long long)kEPT * a.g.thr_x || a.g.thr_x > 256 || a.n_phase > 256 ||
+      !fwd_mode_ok<T>(a.mode))
     return cudaErrorInvalidValue;
   const size_t smem = xpass_smem_bytes(a.g, sizeof(cx<T>));
   auto k = xpass_fwd_kernel<Tf, T, kEptOf<T>>;
@@ -405,7 +406,9 @@ cudaError_t launch_xpass_fwd(const FwdArgs<Tf, T>& a, int nrhs, cudaStream_t s) 
 
 template <typename Tf, typename T>
 cudaError_t launch_xpass_inv(const InvArgs<Tf, T>& a, int nrhs, cudaStream_t s) {
-  if ((long long)a.g.rb * a.g.h > (long long)kEPT * a.g.thr_x || a.g.thr_x > 256) return cudaErrorInvalidValue;
+  if ((long long)a.g.rb * a.g.h > (long long)kEPT * a.g.thr_x || a.g.thr_x > 256 ||
+      !inv_mode_ok<Tf, T>(a.mode))
+    return cudaErrorInvalidValue;
   const size_t smem = xpass_smem_bytes(a.g, sizeof(cx<T>));
   auto k = xpass_inv_kernel<Tf, T, kEptOf<T>>;
   cudaError_t e = set_smem(k, smem);
