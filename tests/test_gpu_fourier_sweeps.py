@@ -1,10 +1,11 @@
-"""What the vectors of FP32 CG and BiCGSTAB in Fourier space must not depend on: the values that earlier calls left in
-their buffers."""
+"""FP32 CG and BiCGSTAB in Fourier space: what earlier calls left in the vectors' buffers does not matter, and
+BiCGSTAB's passes in the launch shapes of larger grids."""
 import numpy as np
 import pytest
 
 from helpers import random_phase
 from paper_1712_05145_gb300 import synthetic
+from test_gpu_spectral_cg import _compare
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -35,3 +36,28 @@ def test_order_1_does_not_read_what_earlier_calls_left_in_the_buffers(grid, sche
         out.append((H.effective(1), [i["iterations"] for i in info]))
         H.close()
     assert out[0][1] == out[1][1] and np.array_equal(out[0][0], out[1][0])
+
+
+@pytest.mark.parametrize("grid,pass_mode", [((128, 128, 96), 0),    # whole planes, wide z tiles, two of them per CTA
+                                            ((128, 128, 96), 2),    # the same by rows and columns
+                                            ((256, 192, 16), 0),    # rows and columns, wide tiles, one per CTA
+                                            ((384, 256, 24), 0),    # ... and three per CTA, odd row blocks
+                                            ((48, 24, 32), 2)],     # narrow tiles, the last one partly past the plane
+                         ids=lambda v: "x".join(map(str, v)) if isinstance(v, tuple) else str(v))
+def test_bicgstab_in_the_launch_shapes_of_larger_grids(grid, pass_mode):
+    from paper_1712_05145_gb300 import hom
+    _compare(grid, pass_mode, hom.HOM_BICGSTAB)
+
+
+@pytest.mark.parametrize("grid", [(32, 24, 16), (128, 96, 128)], ids=lambda g: "x".join(map(str, g)))
+def test_bicgstab_loads_per_launch_do_not_change_the_result(grid):
+    from paper_1712_05145_gb300 import hom
+    out = []
+    for chunk in (1, 6):
+        H = hom.Homogenization(_ms(grid, 5), scheme=hom.HOM_BICGSTAB, rhs_chunk=chunk)
+        info = H.solve(0, 1e-5)
+        assert all(i["status"] == 0 for i in info), info
+        out.append((H.effective(0), H.field(0, 4), [i["iterations"] for i in info]))
+        H.close()
+    assert out[0][2] == out[1][2]
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
