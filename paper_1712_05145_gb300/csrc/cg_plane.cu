@@ -225,8 +225,9 @@ __device__ __forceinline__ int col_rb(int n2) {
 //   2304 to 4608 values: 256 threads of 64 registers, four CTAs: 96^3 0.132 (two of 512 threads: 0.182; three
 //     of 80 registers: 0.148), 128x64x64 0.071 (0.096), 96x48x96 0.078 (0.091)
 //   6144: 256 threads of 80 registers, three CTAs: 128x96x96 0.153 (two of 512: 0.203), 192x64x64 0.125 (0.147)
-//   8192: two CTAs.  128x128x128 gains from 80 registers and 256 threads (0.309, 512 threads of 64: 0.335), the
-//     oblong planes do not (256x64x64 0.181 and 0.170, 64x256x64 0.215 and 0.210)
+//   8192: two CTAs.  Three shapes have that size, and the launch shape is a choice per shape, measured at one depth
+//     and six loads each, not a rule: 128x128 takes 80 registers and 256 threads (128^3 0.309, 512 threads of 64: 0.335),
+//     256x64 and 64x256 keep 512 of 64 (256x64x64 0.181 with 256 of 80, 0.170; 64x256x64 0.215, 0.210)
 // Below 2304 values 8 values per thread are best (32x64x128 0.055, with 256 threads 0.076).
 template <int N2, int H>
 constexpr bool kWidePlane = N2 * H >= 6144 && (N2 * H < kMaxPlane || N2 == 2 * H);   // 80 registers
